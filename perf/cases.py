@@ -84,8 +84,10 @@ def draw(rng):
                        "ba"])
     if kind in ("train", "render", "autograd"):
         w = _log(rng, 96, 1920)
-        c = {"kind": kind, "n": _log(rng, 2000, 500_000), "deg": rng.randint(0, 3), "w": w,
-             "h": max(64, min(1080, int(w * rng.uniform(0.5, 1.0)))), "tile": rng.choice([8, 16, 16, 32])}
+        h = max(64, min(1080, int(w * rng.uniform(0.5, 1.0))))
+        # captures hold at most about one Gaussian per four pixels (the headline workload's density)
+        c = {"kind": kind, "n": _log(rng, 2000, min(500_000, max(2500, w * h // 4))), "deg": rng.randint(0, 3), "w": w,
+             "h": h, "tile": rng.choice([8, 16, 16, 32])}
         if kind == "train":
             c["scene"] = "cloud" if c["n"] <= 4000 else "surface"
             c["dssim"] = rng.choice([0.0, 0.0, 0.2])
