@@ -130,6 +130,17 @@ template <int kDepth>
 struct FwdSmem {
     float4 xyo[kDepth], s2[kDepth], rgb[kDepth];
 };
+// staged entries of the paired-pixel forward, each operand duplicated for the pair's two lanes
+template <int kDepth>
+struct FwdPairSmem {
+    float4 xy[kDepth];  // (u, u, v, v)
+    float4 ab[kDepth];  // (A, A, B, B): base-2 exponent coefficients (scaled conic)
+    float4 co[kDepth];  // (C, C, o, o)
+    float4 rg[kDepth];  // (r, r, g, g)
+    float2 bb[kDepth];  // (b, b)
+};
+template <int kPix, int kDepth>
+using FwdSmemOf = typename std::conditional<kPix == 1, FwdSmem<kDepth>, FwdPairSmem<kDepth>>::type;
 
 // One tile of the forward.  kPix: pixels per thread (vertical strip); kDepth: entries staged per
 // batch.  Every thread of the CTA calls it with the same job.
@@ -542,89 +553,143 @@ __device__ __forceinline__ void pair_alpha(F2 dy, F2 DX, F2 ADX2, F2 S2Y, F2 S2Z
     alpha = make_float2(fminf(kAlphaMax, og.x), fminf(kAlphaMax, og.y));
 }
 
+// The forward is bound by instruction issue and by the ALU and FMA pipes behind it (78 % of the issue
+// slots, ALU 60 %, FMA 48 % before), so a list entry is kept as short as it gets.  Operands both pixels of a pair share are staged twice and load as
+// ready register pairs (three 16-byte loads left eleven moves an entry to form them).  The skip test
+// and the "done" flag are one comparison: a pixel that stopped, or lies outside the image, has an
+// alpha threshold no alpha reaches.  A skipped pixel takes alpha = 0, which leaves its T and colour
+// as they are bit for bit.  Stopping is the rare branch.  The alphas of four list entries
+// are evaluated together: only the transmittance chains them, and a tile with few warps beside it
+// waits on latency.  The composited count of two pixels shares one word: an entry takes at
+// least 1/255 of T and T stays over 1e-4, so no pixel composites more than 2,346 entries.
+// Measured (256 staged): 500k Gaussians at 1920x1080 0.241 -> 0.220 ms, 61k at 1237x693 0.070 -> 0.062,
+// 2k at 128x128 27 -> 24 us; one or two entries at a time take 0.258-0.266 ms at 1920x1080.  The wider
+// staging costs 8-pixel tiles their occupancy at 256 staged entries (0.080 -> 0.092 ms at 100k and
+// 1280x720) (0.061 at 64).
 template <int kT, int kPix, int kDepth>
 __device__ __forceinline__ float2 fwd_tile_pairs(const TileJob& J, int64_t n, const uint32_t* __restrict__ vals,
-                                                 const Scratch& sc, FwdSmem<kDepth>& S) {
+                                                 const Scratch& sc, FwdPairSmem<kDepth>& S) {
     constexpr int kThreads = kT * kT / kPix;
     constexpr int kBatch = kDepth;
     constexpr int NP = kPix / 2;
-    float4* s_xyo = S.xyo;
-    float4* s_s2 = S.s2;
-    float4* s_rgb = S.rgb;
+    constexpr float kNever = 2.0f;  // above every alpha
     const int W = J.W, H = J.H;
     int sdx, sdy0;
     strip_origin<kT, kPix>((int)threadIdx.x, sdx, sdy0);
     const int px = (J.tile % J.TX) * kT + sdx;
     const int py0 = (J.tile / J.TX) * kT + sdy0;
-    const float fx = (float)px + 0.5f;
+    const F2 FX = f2((float)px + 0.5f);
     F2 FY[NP];  // pixel-centre rows of the pairs: dy = row - y exactly as the one-pixel strips
 #pragma unroll
     for (int q = 0; q < NP; ++q) FY[q] = f2((float)(py0 + 2 * q) + 0.5f, (float)(py0 + 2 * q + 1) + 0.5f);
     const uint2 range = J.range;
     const float3 bg = J.bg;
+    const F2 ONE = f2(1.0f);
     F2 T[NP], C0[NP], C1[NP], C2[NP];
-    uint32_t last[kPix], ncomp[kPix];
-    bool done[kPix];
-    bool all_done = true;
+    uint32_t last[kPix], ncomp[NP];
+    float thr[kPix];  // smallest alpha composited: 1/255, or kNever once the pixel is done
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
         T[q] = f2(1.0f);
         C0[q] = C1[q] = C2[q] = f2(0.0f);
+        ncomp[q] = 0;
     }
 #pragma unroll
     for (int k = 0; k < kPix; ++k) {
-        last[k] = ncomp[k] = 0;
-        done[k] = !(px < W && py0 + k < H);
-        all_done = all_done && done[k];
+        last[k] = 0;
+        thr[k] = px < W && py0 + k < H ? kAlphaMin : kNever;
     }
+    auto all_done = [&] {
+        float t = thr[0];
+#pragma unroll
+        for (int k = 1; k < kPix; ++k) t = fminf(t, thr[k]);
+        return t == kNever;
+    };
+    // the alphas of staged entry j at the thread's pixels (the exponent term for term as entry_alpha)
+    auto alphas = [&](int j, float2 (&al)[NP]) {
+        const float4 xy = S.xy[j], ab = S.ab[j], co = S.co[j];
+        const F2 DX = sub2(FX, f2(xy.x, xy.y)), Y = f2(xy.z, xy.w);
+        const F2 ADX2 = mul2(f2(ab.x, ab.y), mul2(DX, DX));
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            float2 G, og;
+            pair_alpha(sub2(FY[q], Y), DX, ADX2, f2(ab.z, ab.w), f2(co.x, co.y), f2(co.z, co.w), G, og, al[q]);
+        }
+    };
+    auto composite = [&](int j, uint32_t pos, const float2 (&al)[NP]) {
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            const int k0 = 2 * q, k1 = 2 * q + 1;
+            bool c0 = al[q].x >= thr[k0], c1 = al[q].y >= thr[k1];
+            if (c0 || c1) {
+                float ax = c0 ? al[q].x : 0.0f, ay = c1 ? al[q].y : 0.0f;
+                F2 Tn = mul2(T[q], sub2(ONE, f2(ax, ay)));
+                const float2 tn = un(Tn);
+                if (fminf(tn.x, tn.y) < kTMin) {  // stop without compositing (T itself is never below)
+                    const float2 tv = un(T[q]);
+                    if (tn.x < kTMin) {
+                        thr[k0] = kNever;
+                        ax = 0.0f;
+                        c0 = false;
+                    }
+                    if (tn.y < kTMin) {
+                        thr[k1] = kNever;
+                        ay = 0.0f;
+                        c1 = false;
+                    }
+                    Tn = f2(tn.x < kTMin ? tv.x : tn.x, tn.y < kTMin ? tv.y : tn.y);
+                }
+                const F2 w = mul2(f2(ax, ay), T[q]);
+                const float4 rg = S.rg[j];
+                const float2 bb = S.bb[j];
+                C0[q] = fma2(f2(rg.x, rg.y), w, C0[q]);
+                C1[q] = fma2(f2(rg.z, rg.w), w, C1[q]);
+                C2[q] = fma2(f2(bb.x, bb.y), w, C2[q]);
+                T[q] = Tn;
+                if (c0) {
+                    last[k0] = pos;
+                    ncomp[q] += 1u;
+                }
+                if (c1) {
+                    last[k1] = pos;
+                    ncomp[q] += 1u << 16;
+                }
+            }
+        }
+    };
     for (uint32_t base = range.x; base < range.y; base += kBatch) {
-        if (__syncthreads_count(all_done) == kThreads) break;
+        if (__syncthreads_count(all_done()) == kThreads) break;
 #pragma unroll
         for (int e = threadIdx.x; e < kBatch; e += kThreads) {
             const uint32_t idx = base + e;
             if (idx < range.y) {
                 const uint32_t id = checked_id(vals[idx], n, sc.status);
-                s_xyo[e] = sc.xyo[id];
-                s_s2[e] = scaled_conic(sc.conic[id]);
-                s_rgb[e] = sc.rgb[id];
+                const float4 p = sc.xyo[id], s2 = scaled_conic(sc.conic[id]), c = sc.rgb[id];
+                S.xy[e] = make_float4(p.x, p.x, p.y, p.y);
+                S.ab[e] = make_float4(s2.x, s2.x, s2.y, s2.y);
+                S.co[e] = make_float4(s2.z, s2.z, p.z, p.z);
+                S.rg[e] = make_float4(c.x, c.x, c.y, c.y);
+                S.bb[e] = make_float2(c.z, c.z);
             }
         }
         __syncthreads();
         const int cnt = min((uint32_t)kBatch, range.y - base);
-        for (int j = 0; !all_done && j < cnt; ++j) {
-            const float4 p = s_xyo[j];
-            const float4 s2 = s_s2[j];
-            const float dx = fx - p.x;
-            const F2 DX = f2(dx), ADX2 = f2(__fmul_rn(s2.x, __fmul_rn(dx, dx)));
-            const F2 S2Y = f2(s2.y), S2Z = f2(s2.z), O = f2(p.z), Y = f2(p.y);
-            const uint32_t pos = base + j - range.x + 1;
-            all_done = true;
+        const uint32_t pos0 = base - range.x + 1;
+        constexpr int kAhead = 4;
+        int j = 0;
+        for (; j + kAhead <= cnt; j += kAhead) {
+            if (__all_sync(kFull, all_done())) break;  // warp-uniform
+            float2 al[kAhead][NP];
 #pragma unroll
-            for (int q = 0; q < NP; ++q) {
-                const int k0 = 2 * q, k1 = 2 * q + 1;
-                const F2 dy = sub2(FY[q], Y);
-                float2 G, og, a;
-                pair_alpha(dy, DX, ADX2, S2Y, S2Z, O, G, og, a);
-                const bool p0 = !done[k0] && a.x >= kAlphaMin, p1 = !done[k1] && a.y >= kAlphaMin;
-                if (p0 || p1) {
-                    const float2 tv = un(T[q]);
-                    const float2 tn = un(mul2(T[q], sub2(f2(1.0f), f2(a.x, a.y))));
-                    const bool s0 = p0 && tn.x < kTMin, s1 = p1 && tn.y < kTMin;  // stop, not composited
-                    const bool c0 = p0 && !s0, c1 = p1 && !s1;
-                    done[k0] = done[k0] || s0;
-                    done[k1] = done[k1] || s1;
-                    const F2 w = mul2(f2(c0 ? a.x : 0.0f, c1 ? a.y : 0.0f), T[q]);
-                    const float4 c = s_rgb[j];
-                    C0[q] = fma2(f2(c.x), w, C0[q]);
-                    C1[q] = fma2(f2(c.y), w, C1[q]);
-                    C2[q] = fma2(f2(c.z), w, C2[q]);
-                    T[q] = f2(c0 ? tn.x : tv.x, c1 ? tn.y : tv.y);
-                    last[k0] = c0 ? pos : last[k0];
-                    last[k1] = c1 ? pos : last[k1];
-                    ncomp[k0] += c0;
-                    ncomp[k1] += c1;
-                }
-                all_done = all_done && done[k0] && done[k1];
+            for (int u = 0; u < kAhead; ++u) alphas(j + u, al[u]);
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) composite(j + u, pos0 + j + u, al[u]);
+        }
+        if (j + kAhead > cnt) {  // the last, shorter group (a warp that broke out has nothing left to do)
+            for (; j < cnt; ++j) {
+                float2 al[NP];
+                alphas(j, al);
+                composite(j, pos0 + j, al);
             }
         }
     }
@@ -645,7 +710,7 @@ __device__ __forceinline__ float2 fwd_tile_pairs(const TileJob& J, int64_t n, co
                 J.image[2 * plane + pp] = ib;
                 J.T_final[pp] = tk[h];
                 J.last[pp] = last[k];
-                J.ncomp[pp] = ncomp[k];
+                J.ncomp[pp] = h ? ncomp[q] >> 16 : ncomp[q] & 0xffffu;
                 if (J.target) l1_pixel(J, pp, plane, ir, ig, ib, l1, l2);
             }
         }
@@ -1234,7 +1299,7 @@ __device__ __forceinline__ void bwd_tile_2p(const TileJob& J, int64_t n, const u
 
 template <int kT, int kPix, int kDepth>
 __device__ __forceinline__ float2 fwd_tile(const TileJob& J, int64_t n, const uint32_t* __restrict__ vals,
-                                           const Scratch& sc, FwdSmem<kDepth>& S) {
+                                           const Scratch& sc, FwdSmemOf<kPix, kDepth>& S) {
     if constexpr (kPix == 1) return fwd_tile_scalar<kT, kPix, kDepth>(J, n, vals, sc, S);
     else return fwd_tile_pairs<kT, kPix, kDepth>(J, n, vals, sc, S);
 }
@@ -1246,7 +1311,7 @@ using BwdSmemOf = typename std::conditional<
     typename std::conditional<kT == 32, BwdSmemPacked<kT, kDepth>, Bwd2Smem<kT, kPix, kDepth>>::type>::type;
 
 template <int kT, int kPix, int kDepth, bool kBackward>
-using BatchSmem = typename std::conditional<kBackward, BwdSmemOf<kT, kPix, kDepth>, FwdSmem<kDepth>>::type;
+using BatchSmem = typename std::conditional<kBackward, BwdSmemOf<kT, kPix, kDepth>, FwdSmemOf<kPix, kDepth>>::type;
 
 // Shared memory of a compositing kernel comes dynamically (the two-phase backward needs more than
 // the 48 KB a static allocation may take); the limit is raised once per kernel.
@@ -1295,7 +1360,7 @@ template <int kT, int kPix, int kDepth>
 __global__ void __launch_bounds__(kT * kT / kPix)
 k_composite_fwd(int W, int H, int TX, float3 bg, int64_t n, const uint32_t* __restrict__ vals,
                 Scratch sc, float* __restrict__ image, int64_t zero_grad, L1Fused l1f) {
-    __shared__ FwdSmem<kDepth> S;
+    __shared__ FwdSmemOf<kPix, kDepth> S;
     TileJob J;
     J.W = W;
     J.H = H;
