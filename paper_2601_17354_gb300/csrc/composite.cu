@@ -1008,11 +1008,22 @@ __device__ __forceinline__ void bwd_tile_sorted(const TileJob& J, int64_t n, con
 // dL/dC>, the colour behind the entry (Eq. 7's C_in) projected on the pixel's upstream gradient:
 // dL/dalpha = T_i (<c_i, dL/dC> - S) and S <- S + alpha_i (<c_i, dL/dC> - S), the recurrence
 // C_in <- C_in (1 - alpha) + alpha c.  A pixel that does not composite an entry takes alpha = 0.
+// Two entries' alphas are evaluated together (only T and S chain the entries).
 //
-// Phase 2 (per entry): the lanes of an entry sum over the warp's pixels the moments
-// sum dpow (1, x, y, x^2, x y, y^2) (pixel centres relative to the tile centre) and
-// sum wgt dL/dC, add them over those lanes and turn them into the nine screen-space gradients:
-// with dx = x - u, dy = y - v,
+// Phase 2 (per round) sums over the warp's pixels the moments sum dpow (1, x, y, x^2, x y, y^2)
+// (pixel centres relative to the tile centre) and sum wgt dL/dC of the round's entries: an
+// [entries x pixels] by [pixels x features] product, on the tensor cores (mma m16n8k8, TF32 operands,
+// FP32 accumulators).  An FP32 factor goes in as two TF32 pieces, the rounded value and the remainder:
+// rows 0-7 of an A tile hold the first pieces of the eight entries' dpow (or wgt), rows 8-15 the second,
+// read from the round's rows as phase 1 left them (one 16-byte load a lane and step); the B tiles are
+// the features (small dyadic numbers, exact in 8 bits, kept as bf16 pairs in registers) and both pieces
+// of dL/dC.  The pieces' sums stay apart and are added in FP32: the parameter gradients' errors against
+// 64 bits are those of the FP32 sums it replaces (7e-7 to 1e-6 on views without decision flips, set by
+// phase 1).  It is bound by issue and latency (14 to 24 warps fit an SM beside 35 to 51 KB a CTA): at
+// 500k Gaussians and 1920x1080 the two phases took 0.503 ms (64 entries staged, 0.546 with 256) with
+// packed FP32 sums over four lanes an entry, 0.471 with the products, 0.451 with the pieces in the
+// tile's two halves instead of two products each (0.133 -> 0.125 ms at 61k and 1237x693).
+// With the moments, dx = x - u, dy = y - v,
 //   sum dpow dx = Mx - u M0,  sum dpow dx^2 = Mxx - 2 u Mx + u^2 M0,  ...,
 //   d mean = (a sum dpow dx + b sum dpow dy, c sum dpow dy + b sum dpow dx),
 //   d conic = -(sum dpow dx^2 / 2, sum dpow dx dy, sum dpow dy^2 / 2),  d opacity = M0 / o,
@@ -1025,27 +1036,48 @@ __device__ __forceinline__ void bwd_tile_sorted(const TileJob& J, int64_t n, con
 // lies inside its pixels' lists with 64 pixels per warp, against 83 % for compact 8 x 8 blocks).
 // Pixel pairs run on the packed f32x2 instructions; every operand that is the same for the pair
 // is staged duplicated, so it loads as a ready pair.
-constexpr int kBwdRound = 8;  // entries per phase-1 / phase-2 round
+constexpr int kBwdRound = 8;  // entries per phase-1 / phase-2 round (rows of half an A tile)
+
+// d += a b with A 16 x 8 (row g = lane / 4: a0, a2; row g + 8: a1, a3; columns t = lane % 4 and t + 4),
+// B 8 x 8 (rows t, t + 4 of column g), D 16 x 8 (columns 2 t, 2 t + 1 of rows g: d0, d1 and g + 8: d2, d3)
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// x as two TF32 pieces: rounded to 11 significant bits (half a unit added, the low 13 bits cut; plain
+// integer instructions, several times cheaper here than cvt.rna.tf32), and the remainder cut to as many
+__device__ __forceinline__ void tf32_split(float x, uint32_t& high, uint32_t& low) {
+    high = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+    low = __float_as_uint(x - __uint_as_float(high)) & 0xffffe000u;
+}
+// x rounded to the nearest TF32 value
+__device__ __forceinline__ float tf32_high(float x) {
+    uint32_t h;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(x));
+    return __uint_as_float(h);
+}
 
 template <int kT, int kPix, int kDepth>
 struct Bwd2Smem {
     static constexpr int kWarps = kT * kT / kPix / 32;
     static constexpr int kPW = 16 * kPix;      // pixel pairs per warp
-    static constexpr int kRow = kPW + 4;       // a round row, padded so that phase 2's reads of two
-                                               // rows fall in different banks
+    static constexpr int kSteps = kPW / 4;     // 8-pixel steps of the phase-2 products
+    static constexpr int kRow = kPW + 4;       // a round row, padded so that the 16-byte reads of a
+                                               // quarter warp (two rows) fall in different banks
     float4 xy[kDepth];  // (u, u, v, v)
     float4 ab[kDepth];  // (A, A, B, B): base-2 exponent coefficients (scaled conic)
     float4 co[kDepth];  // (C, C, o, o)
     float4 rg[kDepth];  // (r, r, g, g) colour
     float4 bz[kDepth];  // (b, b, conic a, conic c) colour blue, conic
     float2 bi[kDepth];  // (conic b, canonical index bits)
-    float4 m0[kWarps * kPW];  // pixel pair (x, x, y, y) relative to the tile centre
-    float4 gg0[kWarps * kPW]; // dL/dC (r, r, g, g)
-    float2 gg1[kWarps * kPW]; // (b, b)
+    float4 gb[kWarps][kSteps / 2][24];  // dL/dC as B fragments: two steps per lane; columns 2 c and
+                                        // 2 c + 1 are the pieces of channel c (6 and 7 are not used)
     uint32_t wmax[32];
-    int rowj[kWarps][kBwdRound];  // staged entry of each row of a warp's round
+    int rowj[kWarps][kBwdRound + 1];  // staged entry of each row of a warp's round
     union {
-        float4 D[kWarps][kBwdRound][kRow];  // per warp, row of the round and pixel pair: (dpow x2, wgt x2)
+        // per warp, row of the round and pixel pair: (dpow x2, wgt x2); an iteration adds up to two rows
+        float4 D[kWarps][kBwdRound + 1][kRow];
         struct {
             uint32_t order[kT * kT];  // tile pixels (row-major index) in the order of their `last`
             uint32_t count[256];
@@ -1057,15 +1089,13 @@ template <int kT, int kPix, int kDepth>
 __device__ __forceinline__ void bwd_tile_2p(const TileJob& J, int64_t n, const uint32_t* __restrict__ vals,
                                             const Scratch& sc, Bwd2Smem<kT, kPix, kDepth>& S) {
     static_assert(kPix == 2 || kPix == 4, "pairs of pixels");
+    static_assert(kT <= 16, "tile-relative features exact in 8 bits");
     using Sm = Bwd2Smem<kT, kPix, kDepth>;
     constexpr int kThreads = kT * kT / kPix;
     constexpr int kWarps = kThreads / 32;
     constexpr int NP = kPix / 2;
-    constexpr int kPW = Sm::kPW;
+    constexpr int kSteps = Sm::kSteps;
     constexpr int kE = kBwdRound;
-    constexpr int L = 32 / kE;       // phase 2: lanes per entry
-    constexpr int kPL = kPW / L;     // pairs per lane
-    static_assert(L >= 1 && (L & (L - 1)) == 0 && kPW % L == 0, "phase-2 lanes");
     const int W = J.W, H = J.H;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int x0 = (J.tile % J.TX) * kT, y0 = (J.tile / J.TX) * kT;
@@ -1117,7 +1147,7 @@ __device__ __forceinline__ void bwd_tile_2p(const TileJob& J, int64_t n, const u
         for (int k = 0; k < kPix; ++k) S.sort.order[atomicAdd(&S.sort.count[bucket[k]], 1u)] = (uint32_t)(tid * kPix + k);
         __syncthreads();
     }
-    // ---- this thread's pixels: kPix consecutive positions of the order = the warp's pairs lane NP + q
+    // ---- this thread's pixels: kPix consecutive positions of the order = the warp's pairs q 32 + lane
     const size_t plane = (size_t)W * H;
     const float3 bg = J.bg;
     F2 FX[NP], FY[NP], T[NP], Sb[NP], g0[NP], g1[NP], g2[NP];
@@ -1152,16 +1182,39 @@ __device__ __forceinline__ void bwd_tile_2p(const TileJob& J, int64_t n, const u
         g2[q] = f2(c[0], c[1]);
         // S = <C_behind, dL/dC>, the background behind the last entry
         Sb[q] = fma2(f2(bg.z), g2[q], fma2(f2(bg.y), g1[q], mul2(f2(bg.x), g0[q])));
-        // the pair's phase-2 operands; pair q of lane l is the warp's pair q 32 + l
-        const int gp = warp * kPW + q * 32 + lane;
-        const float rx0 = fx[0] - cxt, rx1 = fx[1] - cxt, ry0 = fy[0] - cyt, ry1 = fy[1] - cyt;
-        S.m0[gp] = make_float4(rx0, rx1, ry0, ry1);
-        S.gg0[gp] = make_float4(a[0], a[1], b[0], b[1]);
-        S.gg1[gp] = make_float2(c[0], c[1]);
+        // dL/dC of pair p = q 32 + lane: rows t = p % 4 (first pixel) and t + 4 (second) of step p / 4,
+        // columns 2 c (high piece) and 2 c + 1 (remainder) of channel c
+        const int step = (q * 32 + lane) >> 2;
+        float2* const gf = reinterpret_cast<float2*>(&S.gb[warp][step >> 1][lane & 3]) + (step & 1);
+        const float ch[3][2] = {{a[0], a[1]}, {b[0], b[1]}, {c[0], c[1]}};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float h0 = tf32_high(ch[k][0]), h1 = tf32_high(ch[k][1]);
+            gf[8 * (2 * k)] = make_float2(h0, h1);  // lane 4 n + t holds column n: 4 float4 apart
+            gf[8 * (2 * k + 1)] = make_float2(tf32_high(ch[k][0] - h0), tf32_high(ch[k][1] - h1));
+        }
     }
     const uint32_t wmax = __reduce_max_sync(kFull, wlast);
     const F2 ONE = f2(1.0f);
-    const int pe = lane / L, pl = lane % L;  // phase 2: entry of the round, lane inside the entry
+    const int pg = lane >> 2, pt = lane & 3;  // the lane's row and column in the phase-2 products
+    // the features of column pg (1, x, y, x^2, x y, y^2, 0, 0) at the two pixels of pair 4 i + pt, as
+    // the upper halves of FP32 words (exact: at most 8 significant bits)
+    uint32_t feat[kSteps];
+#pragma unroll
+    for (int i = 0; i < kSteps; ++i) {
+        const int q = i / 8, src = (4 * i + pt) & 31;
+        uint32_t packed = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 vx = un(FX[q]), vy = un(FY[q]);
+            const float x = __shfl_sync(kFull, h ? vx.y : vx.x, src) - cxt;
+            const float y = __shfl_sync(kFull, h ? vy.y : vy.x, src) - cyt;
+            const float u = pg == 1 || pg == 3 || pg == 4 ? x : (pg == 2 || pg == 5 ? y : (pg == 0 ? 1.0f : 0.0f));
+            const float v = pg == 3 ? x : (pg == 4 || pg == 5 ? y : 1.0f);
+            packed |= (__float_as_uint(u * v) >> 16) << (16 * h);
+        }
+        feat[i] = packed;
+    }
     float4(* __restrict__ Dw)[Sm::kRow] = S.D[warp];
 
     while (end > 0) {
@@ -1189,109 +1242,121 @@ __device__ __forceinline__ void bwd_tile_2p(const TileJob& J, int64_t n, const u
         // pixel of the warp composites fill rounds of kE rows, each summed by phase 2 when full
         const int jtop = (int)min((uint32_t)cnt, wmax > start ? wmax - start : 0u);
         int nrow = 0;
-        for (int j = jtop - 1; j >= 0; --j) {
-            // ---- phase 1: entry j for this thread's pixels
+        // o G of staged entry j at the thread's pixels (the forward's exponent, term for term)
+        auto evaluate = [&](int j, float2 (&og)[NP]) {
+            const float4 xy = S.xy[j], ab = S.ab[j], co = S.co[j];
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                const F2 DX = sub2(FX[q], f2(xy.x, xy.y)), DY = sub2(FY[q], f2(xy.z, xy.w));
+                const float2 p = un(fma2(f2(co.x, co.y), mul2(DY, DY),
+                                         fma2(f2(ab.z, ab.w), mul2(DX, DY), mul2(f2(ab.x, ab.y), mul2(DX, DX)))));
+                og[q] = un(mul2(f2(co.z, co.w), f2(ex2_approx(p.x), ex2_approx(p.y))));
+            }
+        };
+        // phase 1 of entry j: the pixels' state moves in front of it; it takes the round's next row if
+        // some pixel of the warp composites it
+        auto walk = [&](int j, const float2 (&og)[NP]) {
             const uint32_t pos = start + j;
-            const float4 xy = S.xy[j], ab = S.ab[j], co = S.co[j], rg = S.rg[j], bz = S.bz[j];
-            const F2 X2 = f2(xy.x, xy.y), Y2 = f2(xy.z, xy.w);
-            const F2 A2 = f2(ab.x, ab.y), B2 = f2(ab.z, ab.w), C2 = f2(co.x, co.y), O2 = f2(co.z, co.w);
-            const F2 Cr = f2(rg.x, rg.y), Cg = f2(rg.z, rg.w), Cb = f2(bz.x, bz.y);
-            float4 out1[NP];
+            bool p0[NP], p1[NP];
             bool mine = false;
 #pragma unroll
             for (int q = 0; q < NP; ++q) {
-                const F2 DX = sub2(FX[q], X2), DY = sub2(FY[q], Y2);
-                // the forward's exponent, term for term: A dx^2 + B dx dy + C dy^2
-                const float2 p = un(fma2(C2, mul2(DY, DY), fma2(B2, mul2(DX, DY), mul2(A2, mul2(DX, DX)))));
-                const float2 og = un(mul2(O2, f2(ex2_approx(p.x), ex2_approx(p.y))));
-                const float ax = fminf(kAlphaMax, og.x), ay = fminf(kAlphaMax, og.y);
-                const bool p0 = pos < my_last[2 * q] && ax >= kAlphaMin;
-                const bool p1 = pos < my_last[2 * q + 1] && ay >= kAlphaMin;
-                mine = mine || p0 || p1;
+                p0[q] = pos < my_last[2 * q] && og[q].x >= kAlphaMin;
+                p1[q] = pos < my_last[2 * q + 1] && og[q].y >= kAlphaMin;
+                mine = mine || p0[q] || p1[q];
+            }
+            if (!__any_sync(kFull, mine)) return;  // warp-uniform
+            const float4 rg = S.rg[j];
+            const float2 bb = *reinterpret_cast<const float2*>(&S.bz[j]);
+            const F2 Cr = f2(rg.x, rg.y), Cg = f2(rg.z, rg.w), Cb = f2(bb.x, bb.y);
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
                 // a pixel that does not composite the entry takes alpha = 0
-                const F2 A = f2(p0 ? ax : 0.0f, p1 ? ay : 0.0f);
+                const float ax = p0[q] ? fminf(kAlphaMax, og[q].x) : 0.0f, ay = p1[q] ? fminf(kAlphaMax, og[q].y) : 0.0f;
+                const F2 A = f2(ax, ay);
                 // alpha through which the gradient flows: zero at the 0.99 clamp
-                const F2 AQ = f2(p0 && og.x <= kAlphaMax ? ax : 0.0f, p1 && og.y <= kAlphaMax ? ay : 0.0f);
+                const F2 AQ = f2(og[q].x <= kAlphaMax ? ax : 0.0f, og[q].y <= kAlphaMax ? ay : 0.0f);
                 const float2 om = un(sub2(ONE, A));
                 float rx, ry;
                 asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rx) : "f"(om.x));
                 asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ry) : "f"(om.y));
-                const F2 Tb = mul2(T[q], f2(p0 ? rx : 1.0f, p1 ? ry : 1.0f));  // transmittance in front
+                const F2 Tb = mul2(T[q], f2(p0[q] ? rx : 1.0f, p1[q] ? ry : 1.0f));  // transmittance in front
                 const F2 cg = fma2(Cb, g2[q], fma2(Cg, g1[q], mul2(Cr, g0[q])));
                 const F2 r = sub2(cg, Sb[q]);
                 const float2 dpow = un(mul2(mul2(Tb, r), AQ));
                 const float2 wgt = un(mul2(A, Tb));
                 Sb[q] = fma2(A, r, Sb[q]);
                 T[q] = Tb;
-                out1[q] = make_float4(dpow.x, dpow.y, wgt.x, wgt.y);
+                Dw[nrow][q * 32 + lane] = make_float4(dpow.x, dpow.y, wgt.x, wgt.y);
             }
-            if (__any_sync(kFull, mine)) {  // warp-uniform: the entry gets a row of the round
-#pragma unroll
-                for (int q = 0; q < NP; ++q) Dw[nrow][q * 32 + lane] = out1[q];
-                if (lane == 0) S.rowj[warp][nrow] = j;
-                ++nrow;
+            if (lane == 0) S.rowj[warp][nrow] = j;
+            ++nrow;
+        };
+        int j = jtop - 1;
+        while (j >= 0 || nrow > 0) {  // warp-uniform
+            if (j >= 0) {
+                float2 oga[NP], ogb[NP];
+                evaluate(j, oga);
+                evaluate(max(j - 1, 0), ogb);
+                walk(j, oga);
+                if (j > 0) walk(j - 1, ogb);
+                j -= 2;
             }
-            if (nrow < kE && j > 0) continue;
+            if (nrow < kE && j >= 0) continue;
             if (nrow == 0) break;
             __syncwarp();
-            // ---- phase 2: row pe (entry rowj[pe]), summed over the warp's pairs pl, pl + L, ...
-            // (consecutive lanes read consecutive pairs: no bank conflict)
-            if (pe < nrow) {
-                const float4* __restrict__ Drow = Dw[pe];
-                F2 acc[9];
+            // ---- phase 2: rows 0 .. min(nrow, kE) - 1 of the round, row pg of the A tiles its entry
+            // rowj[pg] (rows past nrow hold earlier rounds' numbers: their sums are not used)
+            float accm[4] = {0.f, 0.f, 0.f, 0.f}, accc[4] = {0.f, 0.f, 0.f, 0.f};
+            const float4* __restrict__ Drow = Dw[pg] + pt;
+            const float4* __restrict__ gf = &S.gb[warp][0][pg < 6 ? lane : lane - 8];
 #pragma unroll
-                for (int k = 0; k < 9; ++k) acc[k] = f2(0.0f);
-#pragma unroll 4
-                for (int k = 0; k < kPL; ++k) {
-                    const int lp = pl + L * k, gp = warp * kPW + lp;
-                    const float4 d = Drow[lp], m0 = S.m0[gp], q0 = S.gg0[gp];
-                    const float2 q1 = S.gg1[gp];
-                    const F2 DP = f2(d.x, d.y), WG = f2(d.z, d.w), X = f2(m0.x, m0.y), Y = f2(m0.z, m0.w);
-                    const F2 DX = mul2(DP, X), DY = mul2(DP, Y);
-                    acc[0] = add2(acc[0], DP);
-                    acc[1] = add2(acc[1], DX);
-                    acc[2] = add2(acc[2], DY);
-                    acc[3] = fma2(DX, X, acc[3]);
-                    acc[4] = fma2(DX, Y, acc[4]);
-                    acc[5] = fma2(DY, Y, acc[5]);
-                    acc[6] = fma2(WG, f2(q0.x, q0.y), acc[6]);
-                    acc[7] = fma2(WG, f2(q0.z, q0.w), acc[7]);
-                    acc[8] = fma2(WG, f2(q1.x, q1.y), acc[8]);
+            for (int i = 0; i < kSteps; i += 2) {
+                const float4 gq = gf[12 * i];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 d = Drow[4 * (i + h)];
+                    uint32_t am[4], ac[4];
+                    tf32_split(d.x, am[0], am[1]);
+                    tf32_split(d.y, am[2], am[3]);
+                    tf32_split(d.z, ac[0], ac[1]);
+                    tf32_split(d.w, ac[2], ac[3]);
+                    mma_tf32(accm, am, feat[i + h] << 16, feat[i + h] & 0xffff0000u);
+                    mma_tf32(accc, ac, __float_as_uint(h ? gq.z : gq.x), __float_as_uint(h ? gq.w : gq.y));
                 }
-                float v[9];
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const float2 h = un(acc[k]);
-                    v[k] = h.x + h.y;
-                }
-                // add over the L lanes of the entry (all of them end with the totals)
-                const unsigned gmask = L == 32 ? kFull : (((1u << L) - 1u) << (lane & ~(L - 1)));
-#pragma unroll
-                for (int o = 1; o < L; o <<= 1)
-#pragma unroll
-                    for (int k = 0; k < 9; ++k) v[k] += __shfl_xor_sync(gmask, v[k], o);
-                const int je = S.rowj[warp][pe];
-                const float M0 = v[0], Mx = v[1], My = v[2], Mxx = v[3], Mxy = v[4], Myy = v[5];
+            }
+            // the pieces' sums: moments 2 pt and 2 pt + 1, and channel pt
+            const float m0 = accm[0] + accm[2], m1 = accm[1] + accm[3];
+            const float col = (accc[0] + accc[1]) + (accc[2] + accc[3]);
+            const int quad = lane & ~3;
+            const float M0 = __shfl_sync(kFull, m0, quad), Mx = __shfl_sync(kFull, m1, quad);
+            const float My = __shfl_sync(kFull, m0, quad + 1), Mxx = __shfl_sync(kFull, m1, quad + 1);
+            const float Mxy = __shfl_sync(kFull, m0, quad + 2), Myy = __shfl_sync(kFull, m1, quad + 2);
+            if (pg < nrow) {
+                const int je = S.rowj[warp][pg];
                 const float u = S.xy[je].x - cxt, vv = S.xy[je].z - cyt;  // mean relative to the tile centre
                 const float sdx = fmaf(-u, M0, Mx), sdy = fmaf(-vv, M0, My);  // sum dpow dx, sum dpow dy
-                float out[9];
                 const float ca = S.bz[je].z, cc = S.bz[je].w, cb = S.bi[je].x;
-                out[0] = fmaf(ca, sdx, cb * sdy);
-                out[1] = fmaf(cc, sdy, cb * sdx);
-                out[2] = -0.5f * fmaf(-u, sdx, fmaf(-u, Mx, Mxx));    // sum dpow dx^2
-                out[3] = -fmaf(-vv, sdx, fmaf(-u, My, Mxy));          // sum dpow dx dy
-                out[4] = -0.5f * fmaf(-vv, sdy, fmaf(-vv, My, Myy));  // sum dpow dy^2
-                out[5] = __fdividef(M0, S.co[je].z);
-                out[6] = v[6];
-                out[7] = v[7];
-                out[8] = v[8];
-                const uint32_t id = __float_as_uint(S.bi[je].y);
-#pragma unroll
-                for (int k = 0; k < 9; ++k)
-                    if (k % L == pl) atomicAdd(&sc.grad2d[(size_t)k * n + id], out[k]);
+                float* const g = sc.grad2d + __float_as_uint(S.bi[je].y);
+                // values pt, 4 + pt (pt < 2) and 6 + pt (pt < 3) of the entry's nine
+                const float v0 = fmaf(ca, sdx, cb * sdy), v1 = fmaf(cc, sdy, cb * sdx);
+                const float v2 = -0.5f * fmaf(-u, sdx, fmaf(-u, Mx, Mxx));    // sum dpow dx^2
+                const float v3 = -fmaf(-vv, sdx, fmaf(-u, My, Mxy));          // sum dpow dx dy
+                const float v4 = -0.5f * fmaf(-vv, sdy, fmaf(-vv, My, Myy));  // sum dpow dy^2
+                const float v5 = __fdividef(M0, S.co[je].z);
+                atomicAdd(g + (size_t)pt * n, pt == 0 ? v0 : (pt == 1 ? v1 : (pt == 2 ? v2 : v3)));
+                if (pt < 2) atomicAdd(g + (size_t)(4 + pt) * n, pt == 0 ? v4 : v5);
+                if (pt < 3) atomicAdd(g + (size_t)(6 + pt) * n, col);
             }
             __syncwarp();
-            nrow = 0;
+            if (nrow > kE) {  // the row past the round starts the next one
+#pragma unroll
+                for (int q = 0; q < NP; ++q) Dw[0][q * 32 + lane] = Dw[kE][q * 32 + lane];
+                if (lane == 0) S.rowj[warp][0] = S.rowj[warp][kE];
+                nrow = 1;
+            } else {
+                nrow = 0;
+            }
         }
         end = start;
     }
