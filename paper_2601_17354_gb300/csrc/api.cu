@@ -39,8 +39,8 @@ struct pgs_ctx {
     int64_t cap_s = 0;
     pgs_camera cam{};
     pgs_gaussians params{};
-    CompositeVariant variant = default_variant();       // forward compositing
-    CompositeVariant variant_bwd = default_variant();   // backward compositing
+    CompositeVariant variant{};      // forward compositing (set at creation)
+    CompositeVariant variant_bwd{};  // backward compositing
     // instrumentation
     int64_t launches = 0;
     bool profiling = false;
@@ -263,6 +263,8 @@ int pgs_create(pgs_ctx** out, const pgs_config* cfg, void* cuda_stream) {
     if (!ctx) return PGS_ERR_OOM;
     ctx->cfg = *cfg;
     ctx->tile = cfg->tile;
+    ctx->variant = default_variant(cfg->tile, false);
+    ctx->variant_bwd = default_variant(cfg->tile, true);
     ctx->stream = static_cast<cudaStream_t>(cuda_stream);
     ctx->grow_pairs = cfg->pair_capacity == 0;
     int rc = reserve_g(ctx, 1, 1, 1, 1);
@@ -784,7 +786,7 @@ struct pgs_batch {
     pgs_gaussians* d_grads = nullptr;  // gradient buffers of pgs_backward_batch, one per scene
     bool rendered = false;             // pgs_render_batch ran since the last parameter change
     int buf = 0;
-    CompositeVariant variant = default_variant();
+    CompositeVariant variant{};  // set at creation
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int64_t launches = 0;
@@ -862,6 +864,7 @@ int pgs_batch_create(pgs_batch** out, const pgs_config* cfg, int32_t n_scenes,
     pgs_batch* b = new (std::nothrow) pgs_batch();
     if (!b) return PGS_ERR_OOM;
     b->cfg = *cfg;
+    b->variant = default_variant(cfg->tile, true);
     b->stream = static_cast<cudaStream_t>(cuda_stream);
     b->S = n_scenes;
     b->R = n_renders;

@@ -565,7 +565,7 @@ __device__ __forceinline__ void pair_alpha(F2 dy, F2 DX, F2 ADX2, F2 S2Y, F2 S2Z
 // Measured (256 staged): 500k Gaussians at 1920x1080 0.241 -> 0.220 ms, 61k at 1237x693 0.070 -> 0.062,
 // 2k at 128x128 27 -> 24 us; one or two entries at a time take 0.258-0.266 ms at 1920x1080.  The wider
 // staging costs 8-pixel tiles their occupancy at 256 staged entries (0.080 -> 0.092 ms at 100k and
-// 1280x720) (0.061 at 64).
+// 1280x720), which is why theirs is 64 (0.061).
 template <int kT, int kPix, int kDepth>
 __device__ __forceinline__ float2 fwd_tile_pairs(const TileJob& J, int64_t n, const uint32_t* __restrict__ vals,
                                                  const Scratch& sc, FwdPairSmem<kDepth>& S) {
@@ -1634,19 +1634,27 @@ __global__ void k_trace_pixels(int W, int H, int TX, int T, int64_t n, const uin
 
 }  // namespace
 
-// pixels per thread and staging depth (64, 128, 256 entries) of the compositing kernels; default
-// (2, 256), the autotuner's choice on the 500k-Gaussian 1080p workload, valid for every tile edge.
-// PGS_COMPOSITE_PIXELS / PGS_COMPOSITE_DEPTH override the default (read once per process).
-CompositeVariant default_variant() {
-    static CompositeVariant v = [] {
-        CompositeVariant c{2, 256};
+// pixels per thread and staging depth (64, 128, 256 entries) of the compositing kernels.  Two pixels
+// everywhere; the depth trades fewer barriers against the CTAs that fit an SM:
+//   edge 8   one warp per CTA: 64 both ways (100k Gaussians, 1280x720: forward 0.061 / 0.071 / 0.092 ms at
+//            64 / 128 / 256, backward 0.131 / 0.153 / 0.227)
+//   edge 16  forward 256 (500k, 1920x1080: 0.226 / 0.220 / 0.220), backward 128 (0.451 / 0.447 / 0.499;
+//            61k, 1237x693: 0.125 / 0.125 / 0.145)
+//   edge 32  256 (not measured apart)
+// A batch has one depth for both directions: the backward's, the longer one.
+// PGS_COMPOSITE_PIXELS / PGS_COMPOSITE_DEPTH override all of them (read once per process).
+CompositeVariant default_variant(int T, bool backward) {
+    static const CompositeVariant env = [] {
+        CompositeVariant c{0, 0};
         if (const char* e = getenv("PGS_COMPOSITE_PIXELS")) c.pix = atoi(e);
         if (const char* e = getenv("PGS_COMPOSITE_DEPTH")) c.depth = atoi(e);
-        if (!valid_variant(c, kTileDefault) || !valid_variant(c, 8) || !valid_variant(c, 32))
-            c = CompositeVariant{2, 256};
+        const CompositeVariant full{c.pix ? c.pix : 2, c.depth ? c.depth : 256};
+        if (!valid_variant(full, kTileDefault) || !valid_variant(full, 8) || !valid_variant(full, 32))
+            c = CompositeVariant{0, 0};
         return c;
     }();
-    return v;
+    const int depth = T == 8 ? 64 : (T == 16 && backward ? 128 : 256);
+    return CompositeVariant{env.pix ? env.pix : 2, env.depth ? env.depth : depth};
 }
 
 // Strips per tile edge: T = 8 takes 1 or 2 pixels per thread (64 or 32 threads per tile), T = 16

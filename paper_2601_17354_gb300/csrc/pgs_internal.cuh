@@ -196,7 +196,7 @@ struct CompositeVariant {
     int pix, depth;
 };
 bool valid_variant(CompositeVariant v, int T);
-CompositeVariant default_variant();
+CompositeVariant default_variant(int T, bool backward);
 
 // ---------------------------------------------------------------------------------------------
 // launchers (all asynchronous on `s`); each returns the number of kernels it launched
