@@ -1210,7 +1210,7 @@ struct pgs_init {
     cudaStream_t stream = nullptr;
     void* scratch = nullptr;
     size_t scratch_bytes = 0;
-    int* bbox = nullptr;
+    uint32_t* tickets = nullptr;  // two arrival counters of the kNN's last-CTA steps, zero between calls
 };
 
 extern "C" {
@@ -1221,8 +1221,10 @@ int pgs_init_create(pgs_init** out, void* cuda_stream) {
     pgs_init* c = new (std::nothrow) pgs_init();
     if (!c) return PGS_ERR_OOM;
     c->stream = static_cast<cudaStream_t>(cuda_stream);
-    const cudaError_t e = cudaMalloc(&c->bbox, 6 * sizeof(int));
+    cudaError_t e = cudaMalloc(&c->tickets, 2 * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->tickets, 0, 2 * sizeof(uint32_t), c->stream);
     if (e != cudaSuccess) {
+        if (c->tickets) cudaFree(c->tickets);
         delete c;
         return cuda_err(e);
     }
@@ -1234,7 +1236,7 @@ void pgs_init_destroy(pgs_init* c) {
     if (!c) return;
     cudaStreamSynchronize(c->stream);
     if (c->scratch) cudaFree(c->scratch);
-    if (c->bbox) cudaFree(c->bbox);
+    if (c->tickets) cudaFree(c->tickets);
     delete c;
 }
 
@@ -1243,17 +1245,10 @@ int pgs_knn(pgs_init* c, const float* points, int64_t n, int32_t k, int32_t* nb)
         return PGS_ERR_INVALID_ARG;
     if (n == 0) return PGS_OK;
     cudaStream_t s = c->stream;
-    launch_bbox(n, points, c->bbox, s);
-    int enc[6];
-    cudaError_t e = cudaMemcpyAsync(enc, c->bbox, sizeof(enc), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_err(e);
-    float bb[6];
-    decode_bbox(enc, bb);
-    // scratch for up to 4 cells per point (the grid coarsens to fit)
-    const size_t want = knn_scratch_bytes(n, 4 * n + 1024);
+    const size_t want = knn_scratch_bytes(n);  // up to 4 cells per point (the grid coarsens to fit)
     if (c->scratch_bytes < want) {
-        e = cudaStreamSynchronize(s);
+        cudaError_t e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return cuda_err(e);
         if (c->scratch) cudaFree(c->scratch);
         c->scratch = nullptr;
         c->scratch_bytes = 0;
@@ -1261,7 +1256,7 @@ int pgs_knn(pgs_init* c, const float* points, int64_t n, int32_t k, int32_t* nb)
         if (e != cudaSuccess) return cuda_err(e);
         c->scratch_bytes = want;
     }
-    launch_knn(n, points, k, nb, c->scratch, c->scratch_bytes, bb, s);
+    launch_knn(n, points, k, nb, c->scratch, c->tickets, s);
     return cuda_err(cudaGetLastError());
 }
 

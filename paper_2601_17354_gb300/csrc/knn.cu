@@ -1,11 +1,13 @@
 // K13 knn_grid and K14 features / PCA initializer (operator I of PocketGS, Sec. III-B).
 //
-// kNN: points are counting-sorted into a uniform grid; each query scans the cells within
-// Chebyshev distance rho of its own cell, keeping a sorted list of its k best (squared distance,
-// index) pairs, and widens rho until the k-th distance is below rho times the cell size, which
-// guarantees that no unscanned point can be closer: the result is the exact k nearest other
-// points.  Squared distances use the fp32 sequence d2 = fma(dx, dx, fma(dy, dy, dz * dz)) with
-// dx = p_j - p_i, ties broken by index, so the neighbour lists are reproducible bit for bit.
+// kNN: points are counting-sorted into a uniform grid whose cells lie row after row, so the cells of a
+// box around a query are a few runs of consecutive points.  A warp takes one query (in cell order, so
+// neighbouring warps read the same runs): its lanes take 32 candidates at a time and hold the K best
+// (squared distance, index) pairs found so far, sorted, one per lane.  The box widens until the
+// k-th distance is below its reach, which guarantees that no point outside can be closer: the result
+// is the exact k nearest other points.  Squared distances use the fp32 sequence
+// d2 = fma(dx, dx, fma(dy, dy, dz * dz)) with dx = p_j - p_i, ties broken by index, so the neighbour
+// lists are reproducible bit for bit.  The bounding box and the grid stay on the device.
 //
 // Features and the paper's initializer are computed per point in FP64 (a few hundred operations
 // per point): Eq. 5 covariance of the K_n = 16 nearest neighbours about their centroid, its
@@ -16,7 +18,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <cstring>
 
 #include "pgs_internal.cuh"
 
@@ -29,39 +30,110 @@ constexpr int kThreads = 256;
 // bits, negative ones flip all but the sign bit, so signed integer order = float order.
 __device__ __host__ __forceinline__ int ordered(int bits) { return bits >= 0 ? bits : bits ^ 0x7fffffff; }
 
-__global__ void k_bbox(int64_t n, const float* __restrict__ P, int* bbox) {
+struct Grid {
+    float lo[3];
+    float h;
+    int dim[3];
+    int cells;
+};
+
+// Is this CTA the last of the grid to get here?  (Its earlier writes are visible to the last one; the
+// last CTA resets the ticket.)  No CTA waits for another.
+__device__ __forceinline__ bool last_cta(uint32_t* ticket) {
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (s_last) *ticket = 0u;
+    }
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
+}
+
+// Bounding box of the points and the grid over it (at most max_cells cells): per-CTA boxes into
+// part [CTAs][6], combined by the last CTA.
+constexpr int kBoxCtas = 152;
+__global__ void __launch_bounds__(kThreads)
+k_bbox(int64_t n, const float* __restrict__ P, float* __restrict__ part, uint32_t* ticket, int64_t max_cells,
+       Grid* __restrict__ grid) {
+    __shared__ float s_box[6][kThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float lo[3] = {3.4e38f, 3.4e38f, 3.4e38f}, hi[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
     for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads)
         for (int d = 0; d < 3; ++d) {
             lo[d] = fminf(lo[d], P[d * n + i]);
             hi[d] = fmaxf(hi[d], P[d * n + i]);
         }
+    auto reduce = [&] {  // over the CTA: thread 0 holds the box
+        for (int d = 0; d < 3; ++d) {
+            for (int o = 16; o > 0; o >>= 1) {
+                lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+                hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+            }
+            if (lane == 0) {
+                s_box[d][warp] = lo[d];
+                s_box[3 + d][warp] = hi[d];
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int d = 0; d < 3; ++d)
+                for (int w = 1; w < kThreads / 32; ++w) {
+                    lo[d] = fminf(lo[d], s_box[d][w]);
+                    hi[d] = fmaxf(hi[d], s_box[3 + d][w]);
+                }
+    };
+    reduce();
+    if (threadIdx.x == 0)
+        for (int d = 0; d < 3; ++d) {
+            part[6 * blockIdx.x + d] = lo[d];
+            part[6 * blockIdx.x + 3 + d] = hi[d];
+        }
+    if (!last_cta(ticket)) return;
     for (int d = 0; d < 3; ++d) {
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
-            hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMin(bbox + d, ordered(__float_as_int(lo[d])));
-            atomicMax(bbox + 3 + d, ordered(__float_as_int(hi[d])));
-        }
+        lo[d] = 3.4e38f;
+        hi[d] = -3.4e38f;
     }
+    for (int c = threadIdx.x; c < (int)gridDim.x; c += kThreads)
+        for (int d = 0; d < 3; ++d) {
+            lo[d] = fminf(lo[d], __ldcg(&part[6 * c + d]));
+            hi[d] = fmaxf(hi[d], __ldcg(&part[6 * c + 3 + d]));
+        }
+    reduce();
+    if (threadIdx.x != 0) return;
+    // cell edge from the bounding box volume per point (the box search keeps it exact whatever the
+    // density): about 2.4 cells per point, so surface points fill few cells densely
+    float e[3];
+    for (int d = 0; d < 3; ++d) e[d] = fmaxf(hi[d] - lo[d], 1e-6f);
+    float h = 0.75f * cbrtf(e[0] * e[1] * e[2] / (float)n);
+    Grid g;
+    for (int tries = 0;; ++tries) {
+        int64_t cells = 1;
+        for (int d = 0; d < 3; ++d) {
+            g.lo[d] = lo[d];
+            // (a box that is not finite, or no edge that fits, ends in one cell)
+            g.dim[d] = tries < 256 && e[d] / h < 3.4e38f ? (int)fminf(1024.f, floorf(e[d] / h) + 1) : 1;
+            cells *= g.dim[d];
+        }
+        g.h = h;
+        g.cells = (int)cells;
+        if (cells <= max_cells) break;
+        h *= 1.25f;
+    }
+    *grid = g;
 }
-
-struct Grid {
-    float lo[3];
-    float h;
-    int dim[3];
-};
 
 __device__ __forceinline__ int cell_coord(float x, float lo, float h, int dim) {
     return min(max((int)floorf((x - lo) / h), 0), dim - 1);
 }
 
-__global__ void k_cell_count(int64_t n, const float* __restrict__ P, Grid g, uint32_t* __restrict__ cell_of,
-                             uint32_t* __restrict__ counts) {
+__global__ void k_cell_count(int64_t n, const float* __restrict__ P, const Grid* __restrict__ grid,
+                             uint32_t* __restrict__ cell_of, uint32_t* __restrict__ counts) {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
+    const Grid g = *grid;
     const int cx = cell_coord(P[i], g.lo[0], g.h, g.dim[0]);
     const int cy = cell_coord(P[n + i], g.lo[1], g.h, g.dim[1]);
     const int cz = cell_coord(P[2 * n + i], g.lo[2], g.h, g.dim[2]);
@@ -70,119 +142,204 @@ __global__ void k_cell_count(int64_t n, const float* __restrict__ P, Grid g, uin
     atomicAdd(&counts[c], 1u);
 }
 
-// exclusive scan of counts[0..m) into start[0..m], start[m] = total (one CTA, chunked)
-__global__ void __launch_bounds__(1024) k_scan_cells(int64_t m, const uint32_t* __restrict__ counts,
-                                                     uint32_t* __restrict__ start) {
-    __shared__ uint32_t s_warp[32];
-    __shared__ uint32_t s_carry;
-    if (threadIdx.x == 0) s_carry = 0;
-    __syncthreads();
+// Exclusive scan of the cells' counts into start [cells + 1] and, in place, into the scatter's cursors:
+// runs of kScanRun cells per CTA, their totals first (the last CTA scans them), then the cells.  One CTA
+// walking all cells took 0.42 ms of the 6.1 ms that 200k points took.
+constexpr int kScanItems = 16;
+constexpr int kScanRun = kThreads * kScanItems;
+
+__device__ __forceinline__ uint32_t cta_exclusive(uint32_t v, uint32_t* s_warp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t base = 0; base < m; base += 1024) {
-        const int64_t idx = base + threadIdx.x;
-        const uint32_t v = idx < m ? counts[idx] : 0u;
-        uint32_t incl = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            const uint32_t w = s_warp[lane];
-            uint32_t wi = w;
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xffffffffu, wi, o);
-                if (lane >= o) wi += t;
-            }
-            s_warp[lane] = wi - w;
-        }
-        __syncthreads();
-        const uint32_t carry = s_carry;
-        if (idx < m) start[idx] = carry + s_warp[warp] + incl - v;
-        __syncthreads();
-        if (threadIdx.x == 1023) s_carry = carry + s_warp[warp] + incl;
-        __syncthreads();
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
     }
-    if (threadIdx.x == 0) start[m] = s_carry;
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    uint32_t before = 0;
+    for (int w = 0; w < warp; ++w) before += s_warp[w];
+    __syncthreads();
+    return before + incl - v;
 }
 
-// points in cell order: their indices and a copy of their positions ([3][n]), so the queries read
-// each cell's candidates contiguously
+__global__ void __launch_bounds__(kThreads)
+k_scan_totals(const Grid* __restrict__ grid, const uint32_t* __restrict__ counts, uint32_t* __restrict__ totals,
+              uint32_t* ticket) {
+    __shared__ uint32_t s_warp[kThreads / 32];
+    __shared__ uint32_t s_carry;
+    const int64_t cells = grid->cells, base = (int64_t)blockIdx.x * kScanRun;
+    uint32_t sum = 0;
+    for (int k = 0; k < kScanItems; ++k) {
+        const int64_t c = base + k * kThreads + threadIdx.x;
+        sum += c < cells ? counts[c] : 0u;
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t t = 0;
+        for (int w = 0; w < kThreads / 32; ++w) t += s_warp[w];
+        totals[blockIdx.x] = t;
+    }
+    if (!last_cta(ticket)) return;
+    if (threadIdx.x == 0) s_carry = 0;
+    __syncthreads();
+    for (int b0 = 0; b0 < (int)gridDim.x; b0 += kThreads) {
+        const int b = b0 + threadIdx.x;
+        const uint32_t v = b < (int)gridDim.x ? __ldcg(&totals[b]) : 0u;
+        const uint32_t carry = s_carry, ex = carry + cta_exclusive(v, s_warp);
+        if (b < (int)gridDim.x) totals[b] = ex;
+        if (threadIdx.x == kThreads - 1) s_carry = ex + v;
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kThreads)
+k_scan_cells(int64_t n, const Grid* __restrict__ grid, uint32_t* __restrict__ counts, const uint32_t* __restrict__ totals,
+             uint32_t* __restrict__ start) {
+    __shared__ uint32_t s_warp[kThreads / 32];
+    const int64_t cells = grid->cells, base = (int64_t)blockIdx.x * kScanRun + threadIdx.x * kScanItems;
+    uint32_t v[kScanItems], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        v[k] = base + k < cells ? counts[base + k] : 0u;
+        sum += v[k];
+    }
+    uint32_t run = totals[blockIdx.x] + cta_exclusive(sum, s_warp);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        if (base + k < cells) start[base + k] = counts[base + k] = run;
+        run += v[k];
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) start[cells] = (uint32_t)n;
+}
+
+// points in cell order: position and index bits in one 16-byte record
 __global__ void k_cell_scatter(int64_t n, const float* __restrict__ P, const uint32_t* __restrict__ cell_of,
-                               uint32_t* __restrict__ cursor, uint32_t* __restrict__ sorted,
-                               float* __restrict__ Ps) {
+                               uint32_t* __restrict__ cursor, float4* __restrict__ Ps) {
     const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
     const uint32_t s = atomicAdd(&cursor[cell_of[i]], 1u);
-    sorted[s] = (uint32_t)i;
-    Ps[s] = P[i];
-    Ps[n + s] = P[n + i];
-    Ps[2 * n + s] = P[2 * n + i];
+    Ps[s] = make_float4(P[i], P[n + i], P[2 * n + i], __int_as_float((int)i));
 }
 
+// One step of a bitonic network over the warp: the lane keeps the smaller of its key and lane ^ j's when
+// `low`, else the larger.
+__device__ __forceinline__ unsigned long long exchange(unsigned long long k, int j, bool low) {
+    const unsigned long long o = __shfl_xor_sync(0xffffffffu, k, j);
+    return (o < k) == low ? o : k;
+}
+
+// The K nearest other points of each point, a warp per point.  Instruction-bound: 32 candidates cost
+// about 40 instructions to fetch and rate, a batch with more than kFew candidates among the best so far
+// one bitonic sort and merge (21 exchanges), fewer of them an insertion each.  A thread per point
+// with its list in registers paid a pass of 32 compare-and-swaps whenever any lane of its warp had
+// a candidate and walked cells one by one: 200k surface points, K = 32, 2.35 ms.
+constexpr int kQueryWarps = 4;
 template <int K>
-__global__ void __launch_bounds__(128)
-k_knn_query(int64_t n, const float* __restrict__ P, Grid g, const uint32_t* __restrict__ start,
-            const uint32_t* __restrict__ sorted, const float* __restrict__ Ps, int32_t* __restrict__ nb) {
-    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
-    if (i >= n) return;
-    const float qx = P[i], qy = P[n + i], qz = P[2 * n + i];
-    const int cx = cell_coord(qx, g.lo[0], g.h, g.dim[0]);
-    const int cy = cell_coord(qy, g.lo[1], g.h, g.dim[1]);
-    const int cz = cell_coord(qz, g.lo[2], g.h, g.dim[2]);
-    float bd[K];
-    int32_t bi[K];
-#pragma unroll
-    for (int a = 0; a < K; ++a) {
-        bd[a] = 3.4e38f;
-        bi[a] = 0x7fffffff;
-    }
+__global__ void __launch_bounds__(32 * kQueryWarps)
+k_knn_query(int64_t n, const Grid* __restrict__ grid, const uint32_t* __restrict__ start, const float4* __restrict__ Ps,
+            int32_t* __restrict__ nb) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kFew = 10;
+    constexpr unsigned long long kNone = ~0ull;
+    const int lane = threadIdx.x & 31;
+    const int64_t s = (int64_t)blockIdx.x * kQueryWarps + (threadIdx.x >> 5);
+    if (s >= n) return;  // the whole warp
+    const Grid g = *grid;
+    const float4 q = Ps[s];
+    const int cx = cell_coord(q.x, g.lo[0], g.h, g.dim[0]);
+    const int cy = cell_coord(q.y, g.lo[1], g.h, g.dim[1]);
+    const int cz = cell_coord(q.z, g.lo[2], g.h, g.dim[2]);
     const int maxr = max(g.dim[0], max(g.dim[1], g.dim[2]));
-    for (int rho = 0; rho <= maxr; ++rho) {
-        for (int dz = -rho; dz <= rho; ++dz) {
-            const int z = cz + dz;
-            if (z < 0 || z >= g.dim[2]) continue;
-            for (int dy = -rho; dy <= rho; ++dy) {
-                const int y = cy + dy;
-                if (y < 0 || y >= g.dim[1]) continue;
-                const bool face = abs(dz) == rho || abs(dy) == rho;
-                for (int dx = -rho; dx <= rho; dx += (face ? 1 : 2 * max(rho, 1))) {
-                    const int x = cx + dx;
-                    if (x < 0 || x >= g.dim[0]) continue;
-                    const uint32_t c = ((uint32_t)z * g.dim[1] + y) * g.dim[0] + x;
-                    for (uint32_t s = start[c]; s < start[c + 1]; ++s) {
-                        const int32_t j = (int32_t)sorted[s];
-                        if (j == i) continue;
-                        const float ex = Ps[s] - qx, ey = Ps[n + s] - qy, ez = Ps[2 * n + s] - qz;
-                        const float d2 = __fmaf_rn(ex, ex, __fmaf_rn(ey, ey, __fmul_rn(ez, ez)));
-                        if (d2 < bd[K - 1] || (d2 == bd[K - 1] && j < bi[K - 1])) {
-                            // insertion by a fixed pass of compare-and-swap (static indices keep the
-                            // list in registers): the candidate trades places with every entry it
-                            // precedes, and the last entry falls off
-                            float cd = d2;
-                            int32_t cj = j;
+    unsigned long long best = kNone;  // lane l: the l-th best key, distance bits << 32 | index
+    int r0 = -1;                      // radius of the box scanned so far
+    int R = 1;
+    for (;;) {
+        // the box of radius R less that of radius r0, as runs of cells along x: a row outside the inner
+        // box is one run, a row through it two
+        const int side = 2 * R + 1, halves = r0 < 0 ? 1 : 2, runs = side * side * halves;
+        for (int base = 0; base < runs; base += 32) {
+            const int run = base + lane, row = run / halves, half = run - row * halves;
+            const int dz = row / side - R, dy = row % side - R;
+            const int y = cy + dy, z = cz + dz;
+            int xa = cx - R, xb = cx + R;
+            if (abs(dy) <= r0 && abs(dz) <= r0) {
+                if (half == 0) xb = cx - r0 - 1;
+                else xa = cx + r0 + 1;
+            } else if (half) {
+                xb = xa - 1;
+            }
+            xa = max(xa, 0);
+            xb = min(xb, g.dim[0] - 1);
+            uint32_t first = 0, cnt = 0;
+            if (run < runs && y >= 0 && y < g.dim[1] && z >= 0 && z < g.dim[2] && xa <= xb) {
+                const uint32_t c = ((uint32_t)z * g.dim[1] + y) * g.dim[0];
+                first = start[c + xa];
+                cnt = start[c + xb + 1] - first;
+            }
+            uint32_t incl = cnt;
 #pragma unroll
-                            for (int a = 0; a < K; ++a) {
-                                const bool before = cd < bd[a] || (cd == bd[a] && cj < bi[a]);
-                                const float td = bd[a];
-                                const int32_t tj = bi[a];
-                                bd[a] = before ? cd : td;
-                                bi[a] = before ? cj : tj;
-                                cd = before ? td : cd;
-                                cj = before ? tj : cj;
-                            }
-                        }
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kAll, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const uint32_t total = __shfl_sync(kAll, incl, 31);
+            const uint32_t shift = first - (incl - cnt);  // candidate k of this run: point shift + k
+            for (uint32_t k0 = 0; k0 < total; k0 += 32) {
+                const uint32_t k = k0 + lane;
+                int lo = 0, hi = 31;  // run of candidate k: the first lane whose inclusive count exceeds k
+#pragma unroll
+                for (int step = 0; step < 5; ++step) {
+                    const int mid = (lo + hi) >> 1;
+                    const uint32_t im = __shfl_sync(kAll, incl, mid);
+                    if (lo < hi) {
+                        if (im > k) hi = mid;
+                        else lo = mid + 1;
                     }
+                }
+                const uint32_t at = __shfl_sync(kAll, shift, lo) + k;
+                unsigned long long key = kNone;
+                if (k < total && at != (uint32_t)s) {
+                    const float4 c = Ps[at];
+                    const float ex = c.x - q.x, ey = c.y - q.y, ez = c.z - q.z;
+                    const float d2 = __fmaf_rn(ex, ex, __fmaf_rn(ey, ey, __fmul_rn(ez, ez)));
+                    if (d2 <= 3.4e38f) key = (unsigned long long)__float_as_uint(d2) << 32 | __float_as_uint(c.w);
+                }
+                unsigned pass = __ballot_sync(kAll, key < __shfl_sync(kAll, best, K - 1));
+                if (__popc(pass) <= kFew) {
+                    for (; pass; pass &= pass - 1u) {
+                        const unsigned long long in = __shfl_sync(kAll, key, __ffs(pass) - 1);
+                        const unsigned long long up = __shfl_up_sync(kAll, best, 1);
+                        if (in < best) best = lane > 0 && up > in ? up : in;
+                    }
+                } else {
+                    // the batch sorted in descending order, the smaller of each lane's two keys, and the
+                    // resulting bitonic sequence merged
+#pragma unroll
+                    for (int w = 2; w <= 32; w <<= 1)
+#pragma unroll
+                        for (int j = w >> 1; j > 0; j >>= 1)
+                            key = exchange(key, j, ((lane & j) == 0) == ((lane & w) != 0 && w < 32));
+                    best = key < best ? key : best;
+#pragma unroll
+                    for (int j = 16; j > 0; j >>= 1) best = exchange(best, j, (lane & j) == 0);
                 }
             }
         }
-        // every point within rho * h of the query lies in the scanned block
-        const float reach = (float)rho * g.h;
-        if (bi[K - 1] != 0x7fffffff && bd[K - 1] < reach * reach * 0.9999f) break;
+        if (R >= maxr) break;  // the whole grid
+        // every point within R h of the query lies in the scanned box
+        const unsigned long long kth = __shfl_sync(kAll, best, K - 1);
+        const float d2 = __uint_as_float((uint32_t)(kth >> 32)), reach = (float)R * g.h;
+        if (kth != kNone && d2 < reach * reach * 0.9999f) break;
+        r0 = R;
+        // the radius the k-th distance asks for, or twice this one while there are fewer than K points
+        R = kth != kNone ? (int)fminf(sqrtf(d2) / g.h * 1.0001f + 1.0f, 1024.f) : 2 * R;
+        R = min(max(R, r0 + 1), maxr);
     }
-#pragma unroll
-    for (int a = 0; a < K; ++a) nb[i * K + a] = bi[a] == 0x7fffffff ? -1 : bi[a];
+    if (lane < K) nb[(int64_t)__float_as_int(q.w) * K + lane] = best == kNone ? -1 : (int32_t)(uint32_t)best;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -440,77 +597,59 @@ int launch_make_targets(int64_t n, const pgs_gaussians& pca, const pgs_gaussians
     return 1;
 }
 
-// Scratch of the kNN: bbox (6 floats), cell of each point (n), counts / cursors (cells + 1),
-// starts (cells + 1), sorted indices (n).  Returns the bytes needed for n points and `cells` cells.
-size_t knn_scratch_bytes(int64_t n, int64_t cells) {
-    return 256 + 4 * (size_t)n + 2 * 4 * (size_t)(cells + 1) + 4 * (size_t)n + 12 * (size_t)n + 5 * 256;
+// Scratch of the kNN for n points and at most `cells` cells: the cell-ordered points, the cell of each
+// point, counts / cursors and starts of the cells, the scan's run totals, the CTAs' boxes, the grid.
+namespace {
+struct KnnScratch {
+    float4* Ps;
+    uint32_t *cell_of, *counts, *start, *totals;
+    float* part;
+    Grid* grid;
+    size_t bytes;
+};
+KnnScratch knn_carve(char* base, int64_t n, int64_t cells) {
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* p = base + off;
+        off += (bytes + 255) & ~(size_t)255;
+        return p;
+    };
+    KnnScratch k;
+    k.Ps = reinterpret_cast<float4*>(take(16 * (size_t)n));
+    k.cell_of = reinterpret_cast<uint32_t*>(take(4 * (size_t)n));
+    k.counts = reinterpret_cast<uint32_t*>(take(4 * (size_t)cells));
+    k.start = reinterpret_cast<uint32_t*>(take(4 * (size_t)(cells + 1)));
+    k.totals = reinterpret_cast<uint32_t*>(take(4 * (size_t)((cells + kScanRun - 1) / kScanRun)));
+    k.part = reinterpret_cast<float*>(take(4 * 6 * kBoxCtas));
+    k.grid = reinterpret_cast<Grid*>(take(sizeof(Grid)));
+    k.bytes = off;
+    return k;
 }
+}  // namespace
 
-int launch_knn(int64_t n, const float* P, int k, int32_t* nb, void* scratch, size_t scratch_bytes,
-               const float* host_bbox, cudaStream_t s) {
+int64_t knn_max_cells(int64_t n) { return std::min<int64_t>(4 * n + 1024, int64_t(1) << 30); }
+size_t knn_scratch_bytes(int64_t n) { return knn_carve(nullptr, n, knn_max_cells(n)).bytes; }
+
+// tickets: two zeroed words, zero again afterwards
+int launch_knn(int64_t n, const float* P, int k, int32_t* nb, void* scratch, uint32_t* tickets, cudaStream_t s) {
     if (n <= 0) return 0;
-    // grid: cell edge from the bounding box volume per point (the ring search keeps it exact
-    // whatever the density)
-    const float ex = fmaxf(host_bbox[3] - host_bbox[0], 1e-6f), ey = fmaxf(host_bbox[4] - host_bbox[1], 1e-6f),
-                ez = fmaxf(host_bbox[5] - host_bbox[2], 1e-6f);
-    // a fine grid (about 2.4 cells per point over the bounding box): surface points fill few
-    // cells densely, and fewer candidates per cell beat fewer, fuller cells
-    float h = 0.75f * cbrtf(ex * ey * ez / (float)n);
-    Grid g;
-    for (int d = 0; d < 3; ++d) g.lo[d] = host_bbox[d];
-    int64_t cells = 0;
-    for (;;) {
-        g.h = h;
-        g.dim[0] = (int)fminf(1024.f, floorf(ex / h) + 1);
-        g.dim[1] = (int)fminf(1024.f, floorf(ey / h) + 1);
-        g.dim[2] = (int)fminf(1024.f, floorf(ez / h) + 1);
-        cells = (int64_t)g.dim[0] * g.dim[1] * g.dim[2];
-        if (knn_scratch_bytes(n, cells) <= scratch_bytes) break;
-        h *= 1.25f;
-    }
-    char* base = static_cast<char*>(scratch);
-    uint32_t* cell_of = reinterpret_cast<uint32_t*>(base + 256);
-    uint32_t* counts = cell_of + n;
-    uint32_t* start = counts + (cells + 1);
-    uint32_t* sorted = start + (cells + 1);
-    float* Ps = reinterpret_cast<float*>(base + ((256 + 4 * (size_t)n + 2 * 4 * (size_t)(cells + 1) +
-                                                   4 * (size_t)n + 255) & ~(size_t)255));
-    cudaMemsetAsync(counts, 0, 4 * (size_t)(cells + 1), s);
+    const int64_t cells = knn_max_cells(n);
+    const KnnScratch w = knn_carve(static_cast<char*>(scratch), n, cells);
+    cudaMemsetAsync(w.counts, 0, 4 * (size_t)cells, s);
     const unsigned blocks = (unsigned)((n + kThreads - 1) / kThreads);
-    k_cell_count<<<blocks, kThreads, 0, s>>>(n, P, g, cell_of, counts);
-    k_scan_cells<<<1, 1024, 0, s>>>(cells, counts, start);
-    cudaMemcpyAsync(counts, start, 4 * (size_t)cells, cudaMemcpyDeviceToDevice, s);
-    k_cell_scatter<<<blocks, kThreads, 0, s>>>(n, P, cell_of, counts, sorted, Ps);
-    const unsigned qb = (unsigned)((n + 127) / 128);
+    const unsigned scans = (unsigned)((cells + kScanRun - 1) / kScanRun);
+    k_bbox<<<std::min(blocks, (unsigned)kBoxCtas), kThreads, 0, s>>>(n, P, w.part, tickets, cells, w.grid);
+    k_cell_count<<<blocks, kThreads, 0, s>>>(n, P, w.grid, w.cell_of, w.counts);
+    k_scan_totals<<<scans, kThreads, 0, s>>>(w.grid, w.counts, w.totals, tickets + 1);
+    k_scan_cells<<<scans, kThreads, 0, s>>>(n, w.grid, w.counts, w.totals, w.start);
+    k_cell_scatter<<<blocks, kThreads, 0, s>>>(n, P, w.cell_of, w.counts, w.Ps);
+    const unsigned qb = (unsigned)((n + kQueryWarps - 1) / kQueryWarps);
     switch (k) {
-        case 3: k_knn_query<3><<<qb, 128, 0, s>>>(n, P, g, start, sorted, Ps, nb); break;
-        case 16: k_knn_query<16><<<qb, 128, 0, s>>>(n, P, g, start, sorted, Ps, nb); break;
-        default: k_knn_query<32><<<qb, 128, 0, s>>>(n, P, g, start, sorted, Ps, nb); break;
+        case 3: k_knn_query<3><<<qb, 32 * kQueryWarps, 0, s>>>(n, w.grid, w.start, w.Ps, nb); break;
+        case 16: k_knn_query<16><<<qb, 32 * kQueryWarps, 0, s>>>(n, w.grid, w.start, w.Ps, nb); break;
+        default: k_knn_query<32><<<qb, 32 * kQueryWarps, 0, s>>>(n, w.grid, w.start, w.Ps, nb); break;
     }
-    return 4;
-}
-
-int launch_bbox(int64_t n, const float* P, int* bbox_dev, cudaStream_t s) {
-    int enc[6];
-    const float inf = 3.4e38f, ninf = -3.4e38f;
-    int bi, bn;
-    memcpy(&bi, &inf, 4);
-    memcpy(&bn, &ninf, 4);
-    for (int d = 0; d < 3; ++d) {
-        enc[d] = ordered(bi);
-        enc[3 + d] = ordered(bn);
-    }
-    cudaMemcpyAsync(bbox_dev, enc, sizeof(enc), cudaMemcpyHostToDevice, s);
-    const int64_t blocks = std::min<int64_t>((n + kThreads - 1) / kThreads, 1024);
-    if (blocks > 0) k_bbox<<<(unsigned)blocks, kThreads, 0, s>>>(n, P, bbox_dev);
-    return 1;
-}
-
-void decode_bbox(const int* enc, float* out) {
-    for (int d = 0; d < 6; ++d) {
-        const int b = ordered(enc[d]);
-        memcpy(&out[d], &b, 4);
-    }
+    return 6;
 }
 
 int launch_features_init(int64_t n, const float* P, const int32_t* nb, float r_normal, float* feats,

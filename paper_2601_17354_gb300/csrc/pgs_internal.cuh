@@ -249,11 +249,8 @@ int launch_bwd_batch(const RenderDesc* renders, const SceneDesc* scenes, int S, 
 int launch_loss_batch(const RenderDesc* renders, int R, int64_t values, double* losses, cudaStream_t s);
 
 // Initializer path (K13 kNN, K14 features + paper initializer, K15 MLP).
-size_t knn_scratch_bytes(int64_t n, int64_t cells);
-int launch_bbox(int64_t n, const float* P, int* bbox_dev, cudaStream_t s);
-void decode_bbox(const int* enc, float* out);
-int launch_knn(int64_t n, const float* P, int k, int32_t* nb, void* scratch, size_t scratch_bytes,
-               const float* host_bbox, cudaStream_t s);
+size_t knn_scratch_bytes(int64_t n);
+int launch_knn(int64_t n, const float* P, int k, int32_t* nb, void* scratch, uint32_t* tickets, cudaStream_t s);
 int launch_features_init(int64_t n, const float* P, const int32_t* nb, float r_normal, float* feats,
                          void* feats_bf16, float* frame_q, pgs_gaussians& init, cudaStream_t s);
 int launch_apply_mlp(int64_t n, const float* y, const pgs_gaussians& pca, pgs_gaussians& out,
