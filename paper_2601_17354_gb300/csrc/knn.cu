@@ -9,12 +9,12 @@
 // d2 = fma(dx, dx, fma(dy, dy, dz * dz)) with dx = p_j - p_i, ties broken by index, so the neighbour
 // lists are reproducible bit for bit.  The bounding box and the grid stay on the device.
 //
-// Features and the paper's initializer are computed per point in FP64 (a few hundred operations
-// per point): Eq. 5 covariance of the K_n = 16 nearest neighbours about their centroid, its
-// smallest-eigenvalue eigenvector as the normal (cyclic Jacobi, eigenvectors canonicalised so the
-// largest-magnitude component is positive), Eq. 6 tangential scale from the K_s = 3 nearest
-// neighbours, normal scale r_normal s_t, z axis rotated onto the normal, opacity logit(0.1); and
-// the 16 features of the learned initializer from the 32 nearest neighbours.
+// Features and the paper's initializer are computed per point at about twice FP32's precision: Eq. 5
+// covariance of the K_n = 16 nearest neighbours about their centroid, its smallest-eigenvalue
+// eigenvector as the normal (cyclic Jacobi, eigenvectors canonicalised so the largest-magnitude
+// component is positive), Eq. 6 tangential scale from the K_s = 3 nearest neighbours, normal scale
+// r_normal s_t, z axis rotated onto the normal, opacity logit(0.1); and the 16 features of the
+// learned initializer from the 32 nearest neighbours.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -343,80 +343,134 @@ k_knn_query(int64_t n, const Grid* __restrict__ grid, const uint32_t* __restrict
 }
 
 // ---------------------------------------------------------------------------------------------
-// features and the paper's initializer (FP64)
+// features and the paper's initializer
 // ---------------------------------------------------------------------------------------------
 
-__device__ void jacobi3(double A[3][3], double w[3], double V[3][3]) {
+// Unevaluated sums of two floats (about 47 bits), by the error-free transformations of Dekker (1971) and
+// Knuth (TAOCP 2, 4.2.2).  GB300 runs FP64 at 1/64 of its FP32 rate, and the eigen-decompositions need
+// well more than 24 bits: nearly flat neighbourhoods lose half of them to the normal.
+struct Df {
+    float h, l;
+};
+__device__ __forceinline__ Df df_fast(float a, float b) {  // |a| >= |b|
+    const float s = __fadd_rn(a, b);
+    return {s, __fadd_rn(b, -__fadd_rn(s, -a))};
+}
+__device__ __forceinline__ Df df_two(float a, float b) {
+    const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
+    return {s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
+}
+__device__ __forceinline__ Df df_add(Df a, Df b) {
+    const Df s = df_two(a.h, b.h), t = df_two(a.l, b.l);
+    const Df u = df_fast(s.h, __fadd_rn(s.l, t.h));
+    return df_fast(u.h, __fadd_rn(u.l, t.l));
+}
+__device__ __forceinline__ Df df_neg(Df a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ Df df_sub(Df a, Df b) { return df_add(a, df_neg(b)); }
+__device__ __forceinline__ Df df_mul(Df a, Df b) {
+    const float p = __fmul_rn(a.h, b.h);
+    return df_fast(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ Df df_scale(Df a, float f) { return {__fmul_rn(a.h, f), __fmul_rn(a.l, f)}; }  // f a power of two
+// a / b rounded to FP32 (both normalised); a zero divisor gives what a.h / b.h gives
+__device__ __forceinline__ float df_ratio(Df a, Df b) {
+    const float q = a.h / b.h;
+    if (!isfinite(q)) return q;
+    const float r = __fadd_rn(__fmaf_rn(-q, b.h, a.h), __fmaf_rn(-q, b.l, a.l));
+    return __fadd_rn(q, r / b.h);
+}
+__device__ __forceinline__ double df_double(Df a) { return (double)a.h + (double)a.l; }
+// |(x, y, z)| to about 45 bits
+__device__ __forceinline__ Df df_norm(Df x, Df y, Df z) {
+    const Df s = df_add(df_add(df_mul(x, x), df_mul(y, y)), df_mul(z, z));
+    if (!(s.h > 0.0f)) return {s.h, 0.0f};
+    const float r = __fsqrt_rn(s.h);
+    const float e = __fadd_rn(__fmaf_rn(-r, r, s.h), s.l);
+    return df_fast(r, __fdividef(0.5f * e, r));
+}
+// one product-sum step: acc += a b, acc kept as a sum and the lost parts' sum (normalised by the caller)
+__device__ __forceinline__ void df_dot(Df& acc, Df a, Df b) {
+    const float p = __fmul_rn(a.h, b.h);
+    const float e = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)));
+    const Df s = df_two(acc.h, p);
+    acc.h = s.h;
+    acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, e));
+}
+
+// Eigen-decomposition of the symmetric matrix (a[0] a[1] a[2]; a[1] a[3] a[4]; a[2] a[4] a[5]) by cyclic
+// Jacobi: w ascending, V columns = eigenvectors with their largest-magnitude component positive.  A
+// rotation's angle needs FP32 only (it leaves the element it clears at 1e-7 of itself, the next sweep
+// at 1e-14); its cosine and sine are formed from that angle to full precision, so V stays orthonormal.
+__device__ void jacobi3(const Df a[6], Df w[3], Df V[3][3]) {
+    Df A[3][3] = {{a[0], a[1], a[2]}, {a[1], a[3], a[4]}, {a[2], a[4], a[5]}};
+#pragma unroll
     for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) V[i][j] = i == j ? 1.0 : 0.0;
-    for (int sweep = 0; sweep < 64; ++sweep) {
-        const double off = A[0][1] * A[0][1] + A[0][2] * A[0][2] + A[1][2] * A[1][2];
-        if (off < 1e-300) break;
-        for (int p = 0; p < 2; ++p)
-            for (int q = p + 1; q < 3; ++q) {
-                if (A[p][q] == 0.0) continue;
-                const double theta = (A[q][q] - A[p][p]) / (2.0 * A[p][q]);
-                const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                const double c = 1.0 / sqrt(t * t + 1.0), s = t * c;
-                for (int k = 0; k < 3; ++k) {
-                    const double akp = A[k][p], akq = A[k][q];
-                    A[k][p] = c * akp - s * akq;
-                    A[k][q] = s * akp + c * akq;
-                }
-                for (int k = 0; k < 3; ++k) {
-                    const double apk = A[p][k], aqk = A[q][k];
-                    A[p][k] = c * apk - s * aqk;
-                    A[q][k] = s * apk + c * aqk;
-                }
-                for (int k = 0; k < 3; ++k) {
-                    const double vkp = V[k][p], vkq = V[k][q];
-                    V[k][p] = c * vkp - s * vkq;
-                    V[k][q] = s * vkp + c * vkq;
-                }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) V[i][j] = {i == j ? 1.0f : 0.0f, 0.0f};
+    const float tiny = 1e-14f * (fabsf(a[0].h) + fabsf(a[3].h) + fabsf(a[5].h));
+#pragma unroll 1
+    for (int sweep = 0; sweep < 10; ++sweep) {
+        if (!(fabsf(A[0][1].h) + fabsf(A[0][2].h) + fabsf(A[1][2].h) > tiny)) break;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const int p = e < 2 ? 0 : 1, q = e == 0 ? 1 : 2, r = 3 - p - q;
+            const Df x = A[p][p], y = A[q][q], z = A[p][q];
+            if (z.h == 0.0f) continue;
+            const float theta = df_sub(y, x).h / (2.0f * z.h);
+            const float t = (theta >= 0.0f ? 1.0f : -1.0f) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.0f)));
+            // c = 1 / sqrt(1 + t^2) by one Newton step from the FP32 value, s = t c
+            const float tt = __fmul_rn(t, t);
+            const Df u = df_two(1.0f, tt);
+            const float ul = __fadd_rn(u.l, __fmaf_rn(t, t, -tt));
+            const float c0 = rsqrtf(u.h), cc0 = __fmul_rn(c0, c0);
+            float err = __fmaf_rn(-u.h, cc0, 1.0f);
+            err = __fmaf_rn(-ul, cc0, __fmaf_rn(-u.h, __fmaf_rn(c0, c0, -cc0), err));
+            const Df c = df_fast(c0, __fmul_rn(0.5f * c0, err)), s = df_mul(c, {t, 0.0f});
+            const Df c2 = df_mul(c, c), s2 = df_mul(s, s), cs = df_mul(c, s);
+            const Df w2 = df_scale(df_mul(cs, z), 2.0f);
+            A[p][p] = df_add(df_sub(df_mul(c2, x), w2), df_mul(s2, y));
+            A[q][q] = df_add(df_add(df_mul(s2, x), w2), df_mul(c2, y));
+            A[p][q] = A[q][p] = df_add(df_mul(cs, df_sub(x, y)), df_mul(df_sub(c2, s2), z));
+            const Df f = A[r][p], g = A[r][q];
+            A[r][p] = A[p][r] = df_sub(df_mul(c, f), df_mul(s, g));
+            A[r][q] = A[q][r] = df_add(df_mul(s, f), df_mul(c, g));
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const Df vp = V[k][p], vq = V[k][q];
+                V[k][p] = df_sub(df_mul(c, vp), df_mul(s, vq));
+                V[k][q] = df_add(df_mul(s, vp), df_mul(c, vq));
             }
+        }
     }
-    int idx[3] = {0, 1, 2};
-    // ascending eigenvalues (three-element sorting network)
-    if (A[idx[1]][idx[1]] < A[idx[0]][idx[0]]) { int t = idx[0]; idx[0] = idx[1]; idx[1] = t; }
-    if (A[idx[2]][idx[2]] < A[idx[1]][idx[1]]) { int t = idx[1]; idx[1] = idx[2]; idx[2] = t; }
-    if (A[idx[1]][idx[1]] < A[idx[0]][idx[0]]) { int t = idx[0]; idx[0] = idx[1]; idx[1] = t; }
-    double W[3][3];
+    auto less = [](Df u, Df v) { return u.h < v.h || (u.h == v.h && u.l < v.l); };
+    // ascending eigenvalues (three-element sorting network over the columns)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) w[k] = A[k][k];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const int i = e == 1 ? 1 : 0, j = i + 1;
+        if (less(w[j], w[i])) {
+            const Df t = w[i];
+            w[i] = w[j];
+            w[j] = t;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const Df v = V[k][i];
+                V[k][i] = V[k][j];
+                V[k][j] = v;
+            }
+        }
+    }
+    auto mag = [](Df v) { return v.h < 0.0f ? df_neg(v) : v; };
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
-        w[k] = A[idx[k]][idx[k]];
-        int big = 0;
-        for (int r = 1; r < 3; ++r)
-            if (fabs(V[r][idx[k]]) > fabs(V[big][idx[k]])) big = r;
-        const double sg = V[big][idx[k]] < 0 ? -1.0 : 1.0;
-        for (int r = 0; r < 3; ++r) W[r][k] = sg * V[r][idx[k]];
+        Df big = V[0][k];
+        if (less(mag(big), mag(V[1][k]))) big = V[1][k];
+        if (less(mag(big), mag(V[2][k]))) big = V[2][k];
+        if (big.h < 0.0f)
+#pragma unroll
+            for (int r = 0; r < 3; ++r) V[r][k] = df_neg(V[r][k]);
     }
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) V[a][b] = W[a][b];
-}
-
-__device__ void neighbour_cov(const float* __restrict__ P, int64_t n, const int32_t* nb, int k, double C[3][3]) {
-    double c[3] = {0, 0, 0};
-    for (int a = 0; a < k; ++a)
-        for (int d = 0; d < 3; ++d) c[d] += P[d * n + nb[a]];
-    for (int d = 0; d < 3; ++d) c[d] /= k;
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) C[a][b] = 0.0;
-    for (int j = 0; j < k; ++j) {
-        double v[3];
-        for (int d = 0; d < 3; ++d) v[d] = P[d * n + nb[j]] - c[d];
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) C[a][b] += v[a] * v[b];
-    }
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) C[a][b] /= k;
-}
-
-__device__ double pdist(const float* __restrict__ P, int64_t n, int64_t i, int64_t j) {
-    double s = 0;
-    for (int d = 0; d < 3; ++d) {
-        const double v = (double)P[d * n + j] - (double)P[d * n + i];
-        s += v * v;
-    }
-    return sqrt(s);
 }
 
 __device__ void mat_to_quat(const double R[3][3], double q[4]) {
@@ -450,59 +504,133 @@ __device__ void mat_to_quat(const double R[3][3], double q[4]) {
 
 // One thread per point: nb [n][32] ascending.  Writes features (fp32 [n][16] and bf16 [n][16]),
 // the eigenframe quaternion frame_q [4][n], and the paper's initializer into init (log-scales,
-// quaternions, opacity logits; means = the points; SH zero).
-__global__ void __launch_bounds__(128)
+// quaternions, opacity logits; means = the points; SH zero).  Each warp first gathers its 32 points'
+// neighbours into shared memory, a point's 32 at a time (one coalesced read of its list), for the two
+// passes over them.  Offsets from the point are exact in two floats and are scaled by a power of two to
+// about 1.  In FP64 throughout, 200k points took 3.33 ms, all of it in the FP64 pipe; FP64 is left
+// where a handful of values a point leave the kernel through a logarithm or a quaternion.
+constexpr int kFeatWarps = 2;
+__global__ void __launch_bounds__(32 * kFeatWarps)
 k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restrict__ nb, float r_normal,
                 float* __restrict__ feats, __nv_bfloat16* __restrict__ feats_bf16, float* __restrict__ frame_q,
                 pgs_gaussians init) {
-    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
-    if (i >= n) return;
-    const int32_t* nbi = nb + i * 32;
-    double C[3][3], w[3], V[3][3];
-    // features from the 32 nearest neighbours
-    neighbour_cov(P, n, nbi, 32, C);
-    jacobi3(C, w, V);
-    float f[16];
-    const double sum = w[0] + w[1] + w[2];
-    for (int a = 0; a < 3; ++a) f[a] = (float)(sum > 0 ? w[a] / sum : 1.0 / 3.0);
-    for (int k = 0; k < 3; ++k)
-        for (int d = 0; d < 3; ++d) f[3 + 3 * k + d] = (float)V[d][k];
-    double md = 0, off[3] = {0, 0, 0};
-    for (int a = 0; a < 32; ++a) {
-        md += pdist(P, n, i, nbi[a]);
-        for (int d = 0; d < 3; ++d) off[d] += (double)P[d * n + nbi[a]] - P[d * n + i];
+    __shared__ float s_nb[kFeatWarps][32][3][33];  // [neighbour][axis][point], padded: gathered by neighbour, read by point
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i0 = ((int64_t)blockIdx.x * kFeatWarps + warp) * 32, i = i0 + lane;
+    for (int p = 0; p < 32 && i0 + p < n; ++p) {
+        const int32_t j = nb[(i0 + p) * 32 + lane];
+        const int64_t k = j >= 0 && j < n ? j : i0 + p;
+        for (int d = 0; d < 3; ++d) s_nb[warp][lane][d][p] = P[d * n + k];
     }
-    md /= 32.0;
-    for (int d = 0; d < 3; ++d) f[12 + d] = (float)(off[d] / 32.0 / md);
-    f[15] = (float)(-3.0 * log(md));
+    __syncwarp();
+    if (i >= n) return;
+    const float p0[3] = {P[i], P[n + i], P[2 * n + i]};
+    // scale: the farthest neighbour's offset has its largest component in [1, 2)
+    float far = 0.f;
+    for (int d = 0; d < 3; ++d) far = fmaxf(far, fabsf(s_nb[warp][31][d][lane] - p0[d]));
+    const int ex = far > 0.f && far < 1e30f ? max(ilogbf(far), -100) : 0;
+    const float scale = ldexpf(1.0f, -ex);
+    auto offset = [&](int a, Df u[3]) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) u[d] = df_scale(df_two(s_nb[warp][a][d][lane], -p0[d]), scale);
+    };
+    // sums of the offsets (the first 16, all 32) and of the distances (the first 3, all 32)
+    const Df zero = {0.f, 0.f};
+    Df m16[3] = {zero, zero, zero}, m32[3] = {zero, zero, zero}, d3 = zero, d32 = zero;
+    for (int a = 0; a < 32; ++a) {
+        Df u[3];
+        offset(a, u);
+        if (a == 16)
+            for (int d = 0; d < 3; ++d) m16[d] = m32[d];
+        if (a == 3) d3 = d32;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) m32[d] = df_add(m32[d], u[d]);
+        d32 = df_add(d32, df_norm(u[0], u[1], u[2]));
+    }
+    // covariances (times 16 and 32) about the means rounded to FP32; the rounding is taken out after
+    float c16[3], c32[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        c16[d] = m16[d].h * 0.0625f;
+        c32[d] = m32[d].h * 0.03125f;
+    }
+    Df C16[6] = {zero, zero, zero, zero, zero, zero}, C32[6] = {zero, zero, zero, zero, zero, zero};
+    auto accumulate = [&](const Df u[3], const float c[3], Df C[6]) {
+        Df v[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const Df t = df_two(u[d].h, -c[d]);
+            v[d] = df_fast(t.h, __fadd_rn(t.l, u[d].l));
+        }
+        int e = 0;
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = x; y < 3; ++y) df_dot(C[e++], v[x], v[y]);
+    };
+    for (int a = 0; a < 32; ++a) {
+        Df u[3];
+        offset(a, u);
+        accumulate(u, c32, C32);
+        if (a < 16) accumulate(u, c16, C16);
+    }
+    // C - k e e^T, e = mean - rounded mean; the division by k scales exactly
+    auto finish = [&](Df C[6], const Df m[3], const float c[3], float inv) {
+        Df e[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) e[d] = df_add(df_scale(m[d], inv), {-c[d], 0.f});
+        int k = 0;
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = x; y < 3; ++y, ++k)
+                C[k] = df_sub(df_scale(df_two(C[k].h, C[k].l), inv), df_mul(e[x], e[y]));
+    };
+    finish(C32, m32, c32, 0.03125f);
+    finish(C16, m16, c16, 0.0625f);
+    Df w[3], V[3][3];
+    jacobi3(C32, w, V);
+    float f[16];
+    const Df sum = df_add(df_add(w[0], w[1]), w[2]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) f[a] = sum.h > 0.f ? df_ratio(w[a], sum) : (float)(1.0 / 3.0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) f[3 + 3 * k + d] = V[d][k].h;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) f[12 + d] = df_ratio(m32[d], d32);
+    const double unit = ldexp(1.0, ex);
+    f[15] = (float)(-3.0 * log(df_double(d32) * (0.03125 * unit)));
+#pragma unroll
     for (int a = 0; a < 16; ++a) {
         feats[i * 16 + a] = f[a];
         feats_bf16[i * 16 + a] = __float2bfloat16_rn(f[a]);
     }
     double R[3][3];
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-        R[d][0] = V[d][2];
-        R[d][1] = V[d][1];
-        R[d][2] = V[d][0];
+        R[d][0] = df_double(V[d][2]);
+        R[d][1] = df_double(V[d][1]);
+        R[d][2] = df_double(V[d][0]);
     }
     const double det = R[0][0] * (R[1][1] * R[2][2] - R[1][2] * R[2][1]) -
                        R[0][1] * (R[1][0] * R[2][2] - R[1][2] * R[2][0]) +
                        R[0][2] * (R[1][0] * R[2][1] - R[1][1] * R[2][0]);
     if (det < 0)
+#pragma unroll
         for (int d = 0; d < 3; ++d) R[d][0] = -R[d][0];
     double q[4];
     mat_to_quat(R, q);
+#pragma unroll
     for (int a = 0; a < 4; ++a) frame_q[a * n + i] = (float)q[a];
 
     // the paper's initializer: normal from 16 neighbours (Eq. 5), scale from 3 (Eq. 6)
-    neighbour_cov(P, n, nbi, 16, C);
-    jacobi3(C, w, V);
-    const double nx = V[0][0], ny = V[1][0], nz = V[2][0];
-    double st = 0;
-    for (int a = 0; a < 3; ++a) st += pdist(P, n, i, nbi[a]);
-    st /= 3.0;
-    init.log_scales[i] = (float)log(st);
-    init.log_scales[n + i] = (float)log(st);
+    jacobi3(C16, w, V);
+    const double nx = df_double(V[0][0]), ny = df_double(V[1][0]), nz = df_double(V[2][0]);
+    const double st = df_double(d3) * unit / 3.0, ls = log(st);
+    init.log_scales[i] = (float)ls;
+    init.log_scales[n + i] = (float)ls;
     init.log_scales[2 * n + i] = (float)log((double)r_normal * st);
     double qw, qx, qy, qz;
     if (nz < -1.0 + 1e-12) {
@@ -519,7 +647,7 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
     init.quats[2 * n + i] = (float)qy;
     init.quats[3 * n + i] = (float)qz;
     init.opacity_logits[i] = (float)log(0.1 / 0.9);
-    for (int d = 0; d < 3; ++d) init.means[d * n + i] = P[d * n + i];
+    for (int d = 0; d < 3; ++d) init.means[d * n + i] = p0[d];
     const int K = (init.sh_degree + 1) * (init.sh_degree + 1);
     for (int c = 0; c < 3 * K; ++c) init.sh[(int64_t)c * n + i] = 0.f;
 }
@@ -655,7 +783,7 @@ int launch_knn(int64_t n, const float* P, int k, int32_t* nb, void* scratch, uin
 int launch_features_init(int64_t n, const float* P, const int32_t* nb, float r_normal, float* feats,
                          void* feats_bf16, float* frame_q, pgs_gaussians& init, cudaStream_t s) {
     if (n <= 0) return 0;
-    k_features_init<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(
+    k_features_init<<<(unsigned)((n + 32 * kFeatWarps - 1) / (32 * kFeatWarps)), 32 * kFeatWarps, 0, s>>>(
         n, P, nb, r_normal, feats, static_cast<__nv_bfloat16*>(feats_bf16), frame_q, init);
     return 1;
 }
