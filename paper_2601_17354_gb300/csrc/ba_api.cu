@@ -14,11 +14,15 @@ struct pgs_ba {
     int64_t* start = nullptr;
     uint32_t* mask = nullptr;
     int64_t *cam_count = nullptr, *cam_start = nullptr, *cam_obs = nullptr;
-    float *Htp = nullptr, *E = nullptr;
-    double *Hpp = nullptr, *bp = nullptr, *Hinv = nullptr, *y = nullptr;
-    double *camp = nullptr, *schp = nullptr, *rhsp = nullptr, *Sfull = nullptr, *rhs = nullptr, *dc = nullptr,
-           *cost = nullptr;
+    float4* Htp = nullptr;  // records of 20 floats
+    float *M = nullptr, *y = nullptr;
+    float2 *Hpp = nullptr, *bp = nullptr, *Hinv = nullptr;  // two-float sums
+    float *camp = nullptr, *schp = nullptr, *rhsp = nullptr, *Sfull = nullptr, *rhs = nullptr;
+    double *dc = nullptr, *cost = nullptr;
     float* Aglob = nullptr;
+    BaCtl* ctl = nullptr;
+    double* costs = nullptr;  // a solve's cost per iteration (grown to iters + 1)
+    int64_t costs_cap = 0;
     float *Rn = nullptr, *tn = nullptr, *Pn = nullptr;
     int* status = nullptr;  // [0] reduced system not positive definite, [1] index check
 };
@@ -78,18 +82,25 @@ int begin(pgs_ba* b, const float* R, const float* t, const int32_t* cam, const i
     return err(cudaGetLastError());
 }
 
-int linearize(pgs_ba* b, const float* R, const float* t, const float* P, const int32_t* cam, const int32_t* pt,
-              const float* uv, const float* K, float sigma, float delta, cudaEvent_t* ev = nullptr) {
-    launch_ba_linearize(b->sh, R, t, P, cam, pt, uv, b->start, b->cam_start, b->cam_obs, K, sigma, delta, b->Htp,
-                        b->Hpp, b->bp, b->camp, b->cost, b->stream, ev);
+struct Problem {  // the caller's arguments of one call
+    const int32_t *cam, *pt;
+    const float *uv, *K;
+    float sigma, delta;
+};
+
+// at (R, t, P); move.R: at the candidate (R, t, P) if it was taken, moving the state
+int linearize(pgs_ba* b, const float* R, const float* t, const float* P, const Problem& q, double* cost,
+              const BaState& move = BaState{}, bool copy_only = false, cudaEvent_t* ev = nullptr) {
+    launch_ba_linearize(b->sh, R, t, P, q.cam, q.pt, q.uv, b->start, b->cam_start, b->cam_obs, q.K, q.sigma, q.delta,
+                        b->Htp, b->Hpp, b->bp, b->camp, cost, b->ctl, move, copy_only, b->stream, ev);
     return err(cudaGetLastError());
 }
 
-void trial(pgs_ba* b, const float* R, const float* t, const float* P, const int32_t* cam, const int32_t* pt, double lam,
-           int axis, float* dcam, float* dP, cudaEvent_t* ev = nullptr) {
-    launch_ba_trial(b->sh, pt, b->start, b->mask, b->cam_start, b->cam_obs, cam, b->Htp, b->Hpp, b->bp, b->camp, lam,
-                    axis, b->Hinv, b->y, b->E, b->schp, b->rhsp, b->Sfull, b->rhs, b->Aglob, b->dc, R, t, P, b->Rn, b->tn, b->Pn, dcam,
-                    dP, b->status, b->stream, ev);
+void trial(pgs_ba* b, const float* R, const float* t, const float* P, const Problem& q, int axis, float* dcam, float* dP,
+           double* cost, cudaEvent_t* ev = nullptr) {
+    launch_ba_trial(b->sh, q.pt, b->start, b->mask, b->cam_start, b->cam_obs, q.cam, q.uv, q.K, q.sigma, q.delta, b->Htp,
+                    b->Hpp, b->bp, b->camp, b->ctl, axis, b->Hinv, b->M, b->y, b->schp, b->rhsp, b->Sfull, b->rhs, b->Aglob,
+                    b->dc, R, t, P, b->Rn, b->tn, b->Pn, dcam, dP, cost, b->status, b->stream, ev);
 }
 
 int finish(pgs_ba* b) {
@@ -118,15 +129,15 @@ int pgs_ba_create(pgs_ba** out, int32_t n_cams, int64_t n_points, int64_t n_obs,
     const BaShape& sh = b->sh;
     const size_t C = n_cams, n = n_points, m = n_obs, N = sh.N;
     const size_t packed = sh.solve_smem ? 1 : N * (N + 1) / 2;
-    const size_t sizes[] = {8 * (n + 1), 4 * sh.W * n, 8 * C, 8 * (C + 1), 8 * m, 4 * 18 * m, 4 * 18 * m,
-                            8 * 6 * n, 8 * 3 * n, 8 * 6 * n, 8 * 3 * n, 8 * 27 * C * sh.chc,
-                            8 * 36 * (size_t)sh.pairs * sh.chs, 8 * 6 * C * sh.chs, 8 * N * N, 8 * N, 4 * packed,
-                            8 * N, 16, 4 * 9 * C, 4 * 3 * C, 4 * 3 * n, 256};
+    const size_t sizes[] = {8 * (n + 1), 4 * sh.W * n, 8 * C * sh.list_blocks, 8 * (C + 1), 8 * m, 4 * 20 * m,
+                            4 * 6 * n, 4 * 3 * n, 8 * 6 * n, 8 * 3 * n, 8 * 6 * n, 4 * 27 * C * sh.chc,
+                            4 * 36 * (size_t)sh.pairs * sh.chs, 4 * 6 * C * sh.chs, 4 * N * N, 4 * N, 4 * packed,
+                            8 * N, 16, sizeof(BaCtl), 4 * 9 * C, 4 * 3 * C, 4 * 3 * n, 256};
     void** slots[] = {(void**)&b->start, (void**)&b->mask, (void**)&b->cam_count, (void**)&b->cam_start,
-                      (void**)&b->cam_obs, (void**)&b->Htp, (void**)&b->E, (void**)&b->Hpp,
-                      (void**)&b->bp, (void**)&b->Hinv, (void**)&b->y, (void**)&b->camp, (void**)&b->schp,
-                      (void**)&b->rhsp, (void**)&b->Sfull, (void**)&b->rhs, (void**)&b->Aglob, (void**)&b->dc, (void**)&b->cost, (void**)&b->Rn,
-                      (void**)&b->tn, (void**)&b->Pn, (void**)&b->status};
+                      (void**)&b->cam_obs, (void**)&b->Htp, (void**)&b->M, (void**)&b->y, (void**)&b->Hpp,
+                      (void**)&b->bp, (void**)&b->Hinv, (void**)&b->camp, (void**)&b->schp, (void**)&b->rhsp,
+                      (void**)&b->Sfull, (void**)&b->rhs, (void**)&b->Aglob, (void**)&b->dc, (void**)&b->cost,
+                      (void**)&b->ctl, (void**)&b->Rn, (void**)&b->tn, (void**)&b->Pn, (void**)&b->status};
     constexpr int kSlots = sizeof(sizes) / sizeof(sizes[0]);
     static_assert(kSlots == sizeof(slots) / sizeof(slots[0]), "one size per buffer");
     size_t total = 0;
@@ -159,6 +170,7 @@ void pgs_ba_destroy(pgs_ba* b) {
     if (!b) return;
     cudaStreamSynchronize(b->stream);
     if (b->arena) cudaFree(b->arena);
+    if (b->costs) cudaFree(b->costs);
     delete b;
 }
 
@@ -176,9 +188,12 @@ int pgs_ba_step(pgs_ba* b, const float* R, const float* t, const float* P, const
         return PGS_ERR_INVALID_ARG;
     int axis = 0;
     int rc = begin(b, R, t, cam, pt, &axis);
-    if (rc == PGS_OK) rc = linearize(b, R, t, P, cam, pt, uv, K, sigma, huber_delta);
     if (rc != PGS_OK) return rc;
-    trial(b, R, t, P, cam, pt, lambda, axis, dcam, dP);
+    const Problem q{cam, pt, uv, K, sigma, huber_delta};
+    launch_ba_begin(lambda, b->ctl, b->cost, b->stream);
+    rc = linearize(b, R, t, P, q, b->cost);
+    if (rc != PGS_OK) return rc;
+    trial(b, R, t, P, q, axis, dcam, dP, nullptr);
     cudaError_t e = cudaMemcpyAsync(cost, b->cost, sizeof(double), cudaMemcpyDeviceToHost, b->stream);
     if (e != cudaSuccess) return err(e);
     return finish(b);
@@ -193,41 +208,37 @@ int pgs_ba_solve(pgs_ba* b, float* R, float* t, float* P, const int32_t* cam, co
     cudaStream_t s = b->stream;
     int axis = 0;
     int rc = begin(b, R, t, cam, pt, &axis);
-    if (rc == PGS_OK) rc = linearize(b, R, t, P, cam, pt, uv, K, sigma, huber_delta);
     if (rc != PGS_OK) return rc;
-    double cur = 0.0;
-    cudaError_t e = cudaMemcpyAsync(&cur, b->cost, sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (iters + 1 > b->costs_cap) {
+        cudaError_t e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return err(e);
+        if (b->costs) cudaFree(b->costs);
+        b->costs = nullptr;
+        b->costs_cap = 0;
+        e = cudaMalloc(&b->costs, sizeof(double) * ((size_t)iters + 1));
+        if (e != cudaSuccess) return err(e);
+        b->costs_cap = (int64_t)iters + 1;
+    }
+    // the whole solve is enqueued; the device accepts or rejects each candidate
+    const Problem q{cam, pt, uv, K, sigma, huber_delta};
+    const BaState state{R, t, P};
+    launch_ba_begin(lambda0, b->ctl, b->cost, s);
+    rc = linearize(b, R, t, P, q, b->cost);
+    launch_ba_decide(true, b->ctl, b->cost, b->status, b->costs, s);
+    for (int it = 0; it < iters && rc == PGS_OK; ++it) {
+        trial(b, R, t, P, q, axis, nullptr, nullptr, b->cost + 1);
+        launch_ba_decide(false, b->ctl, b->cost, b->status, b->costs, s);
+        rc = linearize(b, b->Rn, b->tn, b->Pn, q, nullptr, state, it + 1 == iters);
+    }
+    if (rc != PGS_OK) return rc;
+    BaCtl ctl{};
+    cudaError_t e = cudaMemcpyAsync(&ctl, b->ctl, sizeof(ctl), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(costs, b->costs, sizeof(double) * ((size_t)iters + 1), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return err(e);
-    costs[0] = cur;
-    double lam = lambda0;
-    int acc = 0;
-    for (int it = 0; it < iters; ++it) {
-        trial(b, R, t, P, cam, pt, lam, axis, nullptr, nullptr);
-        launch_ba_cost(b->sh, b->Rn, b->tn, b->Pn, cam, uv, b->start, K, sigma, huber_delta, b->cost + 1, s);
-        double cand = 0.0;
-        int st = 0;
-        e = cudaMemcpyAsync(&cand, b->cost + 1, sizeof(double), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&st, b->status, sizeof(int), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return err(e);
-        if (st) return PGS_ERR_NOT_PD;
-        if (cand < cur) {  // take the candidate and relinearize there
-            cudaMemcpyAsync(R, b->Rn, sizeof(float) * 9 * b->sh.C, cudaMemcpyDeviceToDevice, s);
-            cudaMemcpyAsync(t, b->tn, sizeof(float) * 3 * b->sh.C, cudaMemcpyDeviceToDevice, s);
-            cudaMemcpyAsync(P, b->Pn, sizeof(float) * 3 * b->sh.n, cudaMemcpyDeviceToDevice, s);
-            cur = cand;
-            lam /= 10.0;
-            ++acc;
-            rc = linearize(b, R, t, P, cam, pt, uv, K, sigma, huber_delta);
-            if (rc != PGS_OK) return rc;
-        } else {
-            lam *= 10.0;
-        }
-        costs[it + 1] = cur;
-    }
-    *accepted = acc;
-    return finish(b);
+    if (ctl.stop) return PGS_ERR_NOT_PD;
+    *accepted = ctl.accepted;
+    return PGS_OK;
 }
 
 int pgs_ba_stage_times(pgs_ba* b, const float* R, const float* t, const float* P, const int32_t* cam,
@@ -246,9 +257,11 @@ int pgs_ba_stage_times(pgs_ba* b, const float* R, const float* t, const float* P
         if (e != cudaSuccess) break;
     }
     if (e == cudaSuccess) {
-        linearize(b, R, t, P, cam, pt, uv, K, sigma, huber_delta, ev);
-        trial(b, R, t, P, cam, pt, lambda, axis, nullptr, nullptr, ev + 3);
-        launch_ba_cost(b->sh, b->Rn, b->tn, b->Pn, cam, uv, b->start, K, sigma, huber_delta, b->cost + 1, s);
+        const Problem q{cam, pt, uv, K, sigma, huber_delta};
+        launch_ba_begin(lambda, b->ctl, b->cost, s);
+        linearize(b, R, t, P, q, b->cost, BaState{}, false, ev);
+        trial(b, R, t, P, q, axis, nullptr, nullptr, b->cost + 1, ev + 3);
+        launch_ba_decide(false, b->ctl, b->cost, b->status, b->cost, s);
         cudaEventRecord(ev[7], s);
         e = cudaEventSynchronize(ev[7]);
         for (int k = 0; k < 7 && e == cudaSuccess; ++k) e = cudaEventElapsedTime(&ms[k], ev[k], ev[k + 1]);

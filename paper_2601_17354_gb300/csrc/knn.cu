@@ -19,6 +19,7 @@
 
 #include <algorithm>
 
+#include "df.cuh"
 #include "pgs_internal.cuh"
 
 namespace pgs {
@@ -345,57 +346,6 @@ k_knn_query(int64_t n, const Grid* __restrict__ grid, const uint32_t* __restrict
 // ---------------------------------------------------------------------------------------------
 // features and the paper's initializer
 // ---------------------------------------------------------------------------------------------
-
-// Unevaluated sums of two floats (about 47 bits), by the error-free transformations of Dekker (1971) and
-// Knuth (TAOCP 2, 4.2.2).  GB300 runs FP64 at 1/64 of its FP32 rate, and the eigen-decompositions need
-// well more than 24 bits: nearly flat neighbourhoods lose half of them to the normal.
-struct Df {
-    float h, l;
-};
-__device__ __forceinline__ Df df_fast(float a, float b) {  // |a| >= |b|
-    const float s = __fadd_rn(a, b);
-    return {s, __fadd_rn(b, -__fadd_rn(s, -a))};
-}
-__device__ __forceinline__ Df df_two(float a, float b) {
-    const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
-    return {s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb))};
-}
-__device__ __forceinline__ Df df_add(Df a, Df b) {
-    const Df s = df_two(a.h, b.h), t = df_two(a.l, b.l);
-    const Df u = df_fast(s.h, __fadd_rn(s.l, t.h));
-    return df_fast(u.h, __fadd_rn(u.l, t.l));
-}
-__device__ __forceinline__ Df df_neg(Df a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ Df df_sub(Df a, Df b) { return df_add(a, df_neg(b)); }
-__device__ __forceinline__ Df df_mul(Df a, Df b) {
-    const float p = __fmul_rn(a.h, b.h);
-    return df_fast(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
-}
-__device__ __forceinline__ Df df_scale(Df a, float f) { return {__fmul_rn(a.h, f), __fmul_rn(a.l, f)}; }  // f a power of two
-// a / b rounded to FP32 (both normalised); a zero divisor gives what a.h / b.h gives
-__device__ __forceinline__ float df_ratio(Df a, Df b) {
-    const float q = a.h / b.h;
-    if (!isfinite(q)) return q;
-    const float r = __fadd_rn(__fmaf_rn(-q, b.h, a.h), __fmaf_rn(-q, b.l, a.l));
-    return __fadd_rn(q, r / b.h);
-}
-__device__ __forceinline__ double df_double(Df a) { return (double)a.h + (double)a.l; }
-// |(x, y, z)| to about 45 bits
-__device__ __forceinline__ Df df_norm(Df x, Df y, Df z) {
-    const Df s = df_add(df_add(df_mul(x, x), df_mul(y, y)), df_mul(z, z));
-    if (!(s.h > 0.0f)) return {s.h, 0.0f};
-    const float r = __fsqrt_rn(s.h);
-    const float e = __fadd_rn(__fmaf_rn(-r, r, s.h), s.l);
-    return df_fast(r, __fdividef(0.5f * e, r));
-}
-// one product-sum step: acc += a b, acc kept as a sum and the lost parts' sum (normalised by the caller)
-__device__ __forceinline__ void df_dot(Df& acc, Df a, Df b) {
-    const float p = __fmul_rn(a.h, b.h);
-    const float e = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)));
-    const Df s = df_two(acc.h, p);
-    acc.h = s.h;
-    acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, e));
-}
 
 // Eigen-decomposition of the symmetric matrix (a[0] a[1] a[2]; a[1] a[3] a[4]; a[2] a[4] a[5]) by cyclic
 // Jacobi: w ascending, V columns = eigenvectors with their largest-magnitude component positive.  A

@@ -410,6 +410,7 @@ struct BaShape {
     int N = 0;             // 6 C
     int pairs = 0;         // C (C + 1) / 2 camera pairs
     int chc = 1, chs = 1;  // chunks of a camera's observations in the camera-block and Schur launches
+    int64_t list_blocks = 0;  // blocks of observations in the camera lists' counting sort
     bool blocked = false;  // blocked Cholesky of the full matrix in shared memory (6C <= 224)
     size_t solve_smem = 0; // shared memory of the solve (0: packed matrix in global scratch)
 };
@@ -418,19 +419,34 @@ int ba_configure_solve();
 int launch_ba_check(int64_t m, int64_t n, int C, const int32_t* cam, const int32_t* pt, int* flag, cudaStream_t s);
 int launch_ba_index(const BaShape& sh, const int32_t* pt, const int32_t* cam, int64_t* start, uint32_t* mask,
                     int64_t* cam_count, int64_t* cam_start, int64_t* cam_obs, cudaStream_t s);
+// The control words of a trial or a solve, on the device: damping, the state's cost, whether the last
+// candidate was taken, whether to stop (the reduced system was not positive definite), counters.
+struct BaCtl {
+    double lam, cur;
+    int accept, stop, accepted, it;
+};
+struct BaState {
+    float *R = nullptr, *t = nullptr, *P = nullptr;
+};
+// sets the control words and clears both costs
+int launch_ba_begin(double lam, BaCtl* ctl, double* cost, cudaStream_t s);
+// first: the start's cost cost[0] becomes costs[0]; else accept or reject the candidate of cost cost[1]
+int launch_ba_decide(bool first, BaCtl* ctl, double* cost, const int* status, double* costs, cudaStream_t s);
+// move.R != nullptr: (R, t, P) is the candidate; when ctl says it was taken, it is copied into `move` and
+// linearized there (copy_only: only copied), else nothing happens.  cost may be null.
 int launch_ba_linearize(const BaShape& sh, const float* R, const float* t, const float* P, const int32_t* cam,
                         const int32_t* pt, const float* uv, const int64_t* start, const int64_t* cam_start,
-                        const int64_t* cam_obs, const float K[4], float sigma, float delta, float* Htp, double* Hpp,
-                        double* bp, double* camp, double* cost, cudaStream_t s, cudaEvent_t* ev = nullptr);
+                        const int64_t* cam_obs, const float K[4], float sigma, float delta, float4* Htp, float2* Hpp,
+                        float2* bp, float* camp, double* cost, const BaCtl* ctl, const BaState& move, bool copy_only,
+                        cudaStream_t s, cudaEvent_t* ev = nullptr);
+// one damped step from the linearization: candidate state and its cost (added to *cost; may be null)
 int launch_ba_trial(const BaShape& sh, const int32_t* pt, const int64_t* start, const uint32_t* mask,
-                    const int64_t* cam_start, const int64_t* cam_obs, const int32_t* cam, const float* Htp,
-                    const double* Hpp, const double* bp, const double* camp, double lam, int fixed_axis, double* Hinv,
-                    double* y, float* E, double* schp, double* rhsp, double* Sfull, double* rhs, float* Aglob,
-                    double* dc, const float* R, const float* t, const float* P, float* Rn, float* tn, float* Pn,
-                    float* dcam, float* dP, int* status, cudaStream_t s, cudaEvent_t* ev = nullptr);
-int launch_ba_cost(const BaShape& sh, const float* R, const float* t, const float* P, const int32_t* cam,
-                   const float* uv, const int64_t* start, const float K[4], float sigma, float delta, double* cost,
-                   cudaStream_t s);
+                    const int64_t* cam_start, const int64_t* cam_obs, const int32_t* cam, const float* uv,
+                    const float K[4], float sigma, float delta, const float4* Htp, const float2* Hpp, const float2* bp,
+                    const float* camp, const BaCtl* ctl, int fixed_axis, float2* Hinv, float* M, float* y, float* schp,
+                    float* rhsp, float* Sfull, float* rhs, float* Aglob, double* dc, const float* R, const float* t,
+                    const float* P, float* Rn, float* tn, float* Pn, float* dcam, float* dP, double* cost, int* status,
+                    cudaStream_t s, cudaEvent_t* ev = nullptr);
 int launch_ba_project(int64_t m, int64_t n, int C, const float* R, const float* t, const float* P, const int32_t* cam,
                       const int32_t* pt, const float K[4], float* uv, float* z, cudaStream_t s);
 // Single-reference MVS (Sec. III-A): census, plane maps + cost volume, SGM, selection, fusion,
