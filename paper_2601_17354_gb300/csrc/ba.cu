@@ -147,13 +147,6 @@ __device__ __forceinline__ void jacobians(const float* __restrict__ R, const flo
     }
 }
 
-// sums whose low parts stay unnormalised until the end
-__device__ __forceinline__ void df_acc(Df& s, Df v) {
-    const Df t = df_two(s.h, v.h);
-    s.h = t.h;
-    s.l = __fadd_rn(__fadd_rn(s.l, v.l), t.l);
-}
-__device__ __forceinline__ void df_acc(Df& s, float v) { df_acc(s, Df{v, 0.0f}); }
 // over the kGroup lanes of a point (every lane ends with the sum); `lanes` = the warp's active mask
 template <int kLanes>
 __device__ __forceinline__ void df_lanes_sum(Df& s) {

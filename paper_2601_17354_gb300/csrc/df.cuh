@@ -55,8 +55,20 @@ __device__ __forceinline__ Df df_recip(Df x) {
 }
 // |(x, y, z)|
 __device__ __forceinline__ Df df_norm(Df x, Df y, Df z) {
-    return df_sqrt(df_add(df_add(df_mul(x, x), df_mul(y, y)), df_mul(z, z)));
+    const float a = __fmul_rn(x.h, x.h), b = __fmul_rn(y.h, y.h), c = __fmul_rn(z.h, z.h);
+    const Df s = df_two(a, b), t = df_two(s.h, c);
+    float e = __fadd_rn(__fadd_rn(__fmaf_rn(x.h, x.h, -a), __fmaf_rn(y.h, y.h, -b)), __fmaf_rn(z.h, z.h, -c));
+    const float l = __fmaf_rn(x.h, x.l, __fmaf_rn(y.h, y.l, __fmul_rn(z.h, z.l)));
+    e = __fadd_rn(__fmaf_rn(2.0f, l, e), __fadd_rn(s.l, t.l));
+    return df_sqrt(df_fast(t.h, e));
 }
+// sums whose low parts stay unnormalised until the end
+__device__ __forceinline__ void df_acc(Df& s, Df v) {
+    const Df t = df_two(s.h, v.h);
+    s.h = t.h;
+    s.l = __fadd_rn(__fadd_rn(s.l, v.l), t.l);
+}
+__device__ __forceinline__ void df_acc(Df& s, float v) { df_acc(s, Df{v, 0.0f}); }
 // one product-sum step: acc += a b, acc kept as a sum and the lost parts' sum (normalised by the caller)
 __device__ __forceinline__ void df_dot(Df& acc, Df a, Df b) {
     const float p = __fmul_rn(a.h, b.h);

@@ -458,7 +458,9 @@ __device__ void mat_to_quat(const double R[3][3], double q[4]) {
 // neighbours into shared memory, a point's 32 at a time (one coalesced read of its list), for the two
 // passes over them.  Offsets from the point are exact in two floats and are scaled by a power of two to
 // about 1.  In FP64 throughout, 200k points took 3.33 ms, all of it in the FP64 pipe; FP64 is left
-// where a handful of values a point leave the kernel through a logarithm or a quaternion.
+// where a handful of values a point leave the kernel through a logarithm or a quaternion.  0.39 ms now, with
+// one copy of the eigenvalue code for both neighbourhoods (expanded twice, the code outgrew the
+// instruction cache: 0.46 ms) and one pass over the neighbours for both covariances.
 constexpr int kFeatWarps = 2;
 __global__ void __launch_bounds__(32 * kFeatWarps)
 k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restrict__ nb, float r_normal,
@@ -487,6 +489,7 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
     // sums of the offsets (the first 16, all 32) and of the distances (the first 3, all 32)
     const Df zero = {0.f, 0.f};
     Df m16[3] = {zero, zero, zero}, m32[3] = {zero, zero, zero}, d3 = zero, d32 = zero;
+#pragma unroll 1
     for (int a = 0; a < 32; ++a) {
         Df u[3];
         offset(a, u);
@@ -494,41 +497,46 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
             for (int d = 0; d < 3; ++d) m16[d] = m32[d];
         if (a == 3) d3 = d32;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) m32[d] = df_add(m32[d], u[d]);
-        d32 = df_add(d32, df_norm(u[0], u[1], u[2]));
+        for (int d = 0; d < 3; ++d) df_acc(m32[d], u[d]);
+        df_acc(d32, df_norm(u[0], u[1], u[2]));
     }
-    // covariances (times 16 and 32) about the means rounded to FP32; the rounding is taken out after
-    float c16[3], c32[3];
+    auto settle = [](Df& v) { v = df_two(v.h, v.l); };
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        c16[d] = m16[d].h * 0.0625f;
-        c32[d] = m32[d].h * 0.03125f;
+        settle(m16[d]);
+        settle(m32[d]);
     }
+    settle(d3);
+    settle(d32);
+    // covariances (times 16 and 32) about the 32 neighbours' mean rounded to FP32 in one pass; what the
+    // true means differ by is taken out after
+    float c32[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) c32[d] = m32[d].h * 0.03125f;
     Df C16[6] = {zero, zero, zero, zero, zero, zero}, C32[6] = {zero, zero, zero, zero, zero, zero};
-    auto accumulate = [&](const Df u[3], const float c[3], Df C[6]) {
-        Df v[3];
+#pragma unroll 1
+    for (int a = 0; a < 32; ++a) {
+        Df u[3], v[3];
+        offset(a, u);
+        if (a == 16)
+#pragma unroll
+            for (int e = 0; e < 6; ++e) C16[e] = C32[e];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const Df t = df_two(u[d].h, -c[d]);
+            const Df t = df_two(u[d].h, -c32[d]);
             v[d] = df_fast(t.h, __fadd_rn(t.l, u[d].l));
         }
         int e = 0;
 #pragma unroll
         for (int x = 0; x < 3; ++x)
 #pragma unroll
-            for (int y = x; y < 3; ++y) df_dot(C[e++], v[x], v[y]);
-    };
-    for (int a = 0; a < 32; ++a) {
-        Df u[3];
-        offset(a, u);
-        accumulate(u, c32, C32);
-        if (a < 16) accumulate(u, c16, C16);
+            for (int y = x; y < 3; ++y) df_dot(C32[e++], v[x], v[y]);
     }
-    // C - k e e^T, e = mean - rounded mean; the division by k scales exactly
-    auto finish = [&](Df C[6], const Df m[3], const float c[3], float inv) {
+    // C - k e e^T, e = mean - centre; the division by k scales exactly
+    auto finish = [&](Df C[6], const Df m[3], float inv) {
         Df e[3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) e[d] = df_add(df_scale(m[d], inv), {-c[d], 0.f});
+        for (int d = 0; d < 3; ++d) e[d] = df_add(df_scale(m[d], inv), {-c32[d], 0.f});
         int k = 0;
 #pragma unroll
         for (int x = 0; x < 3; ++x)
@@ -536,10 +544,21 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
             for (int y = x; y < 3; ++y, ++k)
                 C[k] = df_sub(df_scale(df_two(C[k].h, C[k].l), inv), df_mul(e[x], e[y]));
     };
-    finish(C32, m32, c32, 0.03125f);
-    finish(C16, m16, c16, 0.0625f);
-    Df w[3], V[3][3];
-    jacobi3(C32, w, V);
+    finish(C32, m32, 0.03125f);
+    finish(C16, m16, 0.0625f);
+    // both decompositions through one copy of the code: it and the loops above are several times the
+    // instruction cache when expanded
+    Df w[3], V[3][3], nrm[3];
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        Df C[6];
+#pragma unroll
+        for (int e = 0; e < 6; ++e) C[e] = pass ? C32[e] : C16[e];
+        jacobi3(C, w, V);
+        if (pass == 0)  // the smallest eigenvector of the 16 neighbours: the normal
+#pragma unroll
+            for (int d = 0; d < 3; ++d) nrm[d] = V[d][0];
+    }
     float f[16];
     const Df sum = df_add(df_add(w[0], w[1]), w[2]);
 #pragma unroll
@@ -576,8 +595,7 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
     for (int a = 0; a < 4; ++a) frame_q[a * n + i] = (float)q[a];
 
     // the paper's initializer: normal from 16 neighbours (Eq. 5), scale from 3 (Eq. 6)
-    jacobi3(C16, w, V);
-    const double nx = df_double(V[0][0]), ny = df_double(V[1][0]), nz = df_double(V[2][0]);
+    const double nx = df_double(nrm[0]), ny = df_double(nrm[1]), nz = df_double(nrm[2]);
     const double st = df_double(d3) * unit / 3.0, ls = log(st);
     init.log_scales[i] = (float)ls;
     init.log_scales[n + i] = (float)ls;
