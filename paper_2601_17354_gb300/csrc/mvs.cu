@@ -34,8 +34,7 @@ __device__ __forceinline__ float luma(float r, float g, float b) {
     return __fadd_rn(__fadd_rn(__fmul_rn(0.299f, r), __fmul_rn(0.587f, g)), __fmul_rn(0.114f, b));
 }
 
-__global__ void __launch_bounds__(kCtx * kCty)
-k_census(const float* __restrict__ rgb, int W, int H, uint64_t* __restrict__ code) {
+__device__ void census_tile(const float* __restrict__ rgb, int W, int H, uint64_t* __restrict__ code) {
     __shared__ float s[kCty + 2 * kR][kCtx + 2 * kR];
     const int x0 = blockIdx.x * kCtx, y0 = blockIdx.y * kCty;
     const size_t plane = (size_t)W * H;
@@ -86,10 +85,8 @@ __device__ __forceinline__ double dsub(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double ddiv(double a, double b) { return __ddiv_rn(a, b); }
 
-// plane maps H_k (FP64 in the order of the definition, rounded to FP32), thread per plane
-__global__ void k_plane_maps(CamF t, CamF r, double inv_far, double step, int D, float* __restrict__ maps) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= D) return;
+// plane map H_k (FP64 in the order of the definition, rounded to FP32)
+__device__ void plane_map(const CamF& t, const CamF& r, double inv_far, double step, int k, float* __restrict__ maps) {
     double Rt[3][3], tt[3], Rr[3][3], tr[3];
     for (int i = 0; i < 3; ++i) {
         for (int j = 0; j < 3; ++j) {
@@ -124,170 +121,249 @@ __global__ void k_plane_maps(CamF t, CamF r, double inv_far, double step, int D,
     }
 }
 
-// cost volume: CTA = D threads (thread k = plane k, its map in registers) over a run of pixels
+// Census codes of both images (blockIdx.z = 0 target, 1 reference) and, in the first CTA's row of a third
+// layer, the plane maps, a thread per plane: they wait for nothing, so they take no launch of their own.
+__global__ void __launch_bounds__(kCtx * kCty)
+k_census(const float* __restrict__ rgb_t, const float* __restrict__ rgb_r, int W, int H, uint64_t* __restrict__ code_t,
+         uint64_t* __restrict__ code_r, CamF t, CamF r, double inv_far, double step, int D, float* __restrict__ maps) {
+    if (blockIdx.z == 2) {
+        const int k = threadIdx.y * kCtx + threadIdx.x;
+        if (blockIdx.x == 0 && blockIdx.y == 0 && k < D) plane_map(t, r, inv_far, step, k, maps);
+        return;
+    }
+    census_tile(blockIdx.z ? rgb_r : rgb_t, W, H, blockIdx.z ? code_r : code_t);
+}
+
+// The integer nearest q - 1/2, which is floor(q) unless an integer lies within the margin (then `sure` turns
+// false): rounding by adding 1.5 2^23, since conversions run at an eighth of the rate.
+__device__ __forceinline__ int floor_fast(float q, bool& sure) {
+    const float m = __fadd_rn(q, -0.5f), t = __fadd_rn(m, 12582912.0f);
+    const float d = __fadd_rn(m, -__fadd_rn(t, -12582912.0f));
+    // (also false for |q| over 2^18 and for NaN)
+    sure = sure && fabsf(d) < __fmaf_rn(fabsf(q), -1e-6f, 0.499998f);
+    return __float_as_int(t) - 0x4b400000;
+}
+
+// Cost volume: CTA = D threads (thread k = plane k, its map in registers) over a run of pixels.  Bound by
+// instruction issue.  The reference pixel is the floor of a correctly rounded quotient; the
+// quotient by the approximate reciprocal is within 4e-7 of itself of that, so only where an integer
+// lies nearer do the divisions decide (a warp in thirty or so).  14.7 M pixels and planes: 43 us with both
+// divisions always, 34 us now.
 __global__ void k_cost(const uint64_t* __restrict__ cen_t, const uint64_t* __restrict__ cen_r, int W, int H,
                        int D, const float* __restrict__ maps, uint8_t* __restrict__ C) {
     const int k = threadIdx.x;
-    const int y = blockIdx.y, xs = blockIdx.x * kRun;
+    const int y = blockIdx.y, xs = blockIdx.x * kRun, xe = min(xs + kRun, W);
     float h[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) h[q] = maps[9 * k + q];
-    const float fW = (float)W, fH = (float)H;
     const float yc = (float)y + 0.5f;
-    for (int x = xs; x < xs + kRun && x < W; ++x) {
-        const float xc = (float)x + 0.5f;
-        const float a = __fadd_rn(__fadd_rn(__fmul_rn(h[0], xc), __fmul_rn(h[1], yc)), h[2]);
-        const float b = __fadd_rn(__fadd_rn(__fmul_rn(h[3], xc), __fmul_rn(h[4], yc)), h[5]);
-        const float c = __fadd_rn(__fadd_rn(__fmul_rn(h[6], xc), __fmul_rn(h[7], yc)), h[8]);
+    const float hy[3] = {__fmul_rn(h[1], yc), __fmul_rn(h[4], yc), __fmul_rn(h[7], yc)};
+    const uint64_t* __restrict__ row = cen_t + (size_t)y * W;
+    uint8_t* __restrict__ out = C + ((size_t)y * W + xs) * D + k;
+    float xc = (float)xs + 0.5f;
+#pragma unroll 2
+    for (int x = xs; x < xe; ++x, xc += 1.0f, out += D) {
+        const float a = __fadd_rn(__fadd_rn(__fmul_rn(h[0], xc), hy[0]), h[2]);
+        const float b = __fadd_rn(__fadd_rn(__fmul_rn(h[3], xc), hy[1]), h[5]);
+        const float c = __fadd_rn(__fadd_rn(__fmul_rn(h[6], xc), hy[2]), h[8]);
         int cost = kInvalid;
         if (c > 0.f) {
-            const float u = __fdiv_rn(a, c), v = __fdiv_rn(b, c);
-            if (u >= 0.f && u < fW && v >= 0.f && v < fH) {
-                const int iu = (int)floorf(u), iv = (int)floorf(v);
-                cost = __popcll(cen_t[(size_t)y * W + x] ^ cen_r[(size_t)iv * W + iu]);
+            float rc;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(c));
+            bool sure = c > 1e-30f && c < 1e30f;
+            int iu = floor_fast(__fmul_rn(a, rc), sure), iv = floor_fast(__fmul_rn(b, rc), sure);
+            if (!sure) {
+                const float u = __fdiv_rn(a, c), v = __fdiv_rn(b, c);
+                const bool in = u >= 0.f && u < (float)W && v >= 0.f && v < (float)H;
+                iu = in ? (int)floorf(u) : -1;
+                iv = in ? (int)floorf(v) : -1;
             }
+            if ((unsigned)iu < (unsigned)W && (unsigned)iv < (unsigned)H)
+                cost = __popcll(__ldg(row + x) ^ __ldg(cen_r + (iv * W + iu)));  // W H <= 2^28
         }
-        C[((size_t)y * W + x) * D + k] = (uint8_t)cost;
+        *out = (uint8_t)cost;
     }
+}
+
+// A lane's KPL consecutive bytes of a pixel's D costs, as one word: one access when D is a multiple of
+// KPL (then every lane's bytes are aligned to themselves, and lanes past D read nothing).
+template <int KPL, bool kVec>
+__device__ __forceinline__ uint32_t load_bytes(const uint8_t* __restrict__ p, int k0, int D) {
+    if constexpr (kVec) {
+        if (k0 >= D) return 0u;
+        if constexpr (KPL == 1) return __ldg(p);
+        if constexpr (KPL == 2) return __ldg(reinterpret_cast<const uint16_t*>(p));
+        if constexpr (KPL == 4) return __ldg(reinterpret_cast<const uint32_t*>(p));
+    }
+    uint32_t v = 0;
+#pragma unroll
+    for (int j = 0; j < KPL; ++j)
+        if (k0 + j < D) v |= (uint32_t)__ldg(p + j) << (8 * j);
+    return v;
+}
+template <int KPL, bool kVec>
+__device__ __forceinline__ void store_bytes(uint8_t* __restrict__ p, int k0, int D, uint32_t v) {
+    if constexpr (kVec) {
+        if (k0 >= D) return;
+        if constexpr (KPL == 1) *p = (uint8_t)v;
+        if constexpr (KPL == 2) *reinterpret_cast<uint16_t*>(p) = (uint16_t)v;
+        if constexpr (KPL == 4) *reinterpret_cast<uint32_t*>(p) = v;
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < KPL; ++j)
+        if (k0 + j < D) p[j] = (uint8_t)(v >> (8 * j));
 }
 
 // the four SGM paths in one launch (blockIdx.y = direction: 0 left to right, 1 right to left,
 // 2 top down, 3 bottom up), warp per scanline, lane holding planes lane * KPL .. + KPL - 1; each
-// path writes its own L (<= 48 + P2 = 80, a byte) so the directions run concurrently, and the
-// costs of the next steps are loaded ahead (the walk along a line is the only serial part)
-template <int KPL>
-__global__ void __launch_bounds__(128)
+// path writes its own L (<= 48 + P2 = 80, a byte) so the directions run concurrently.  The walk along a
+// line is serial: a step waits for the warp's minimum and two shuffles.  The costs of kBatch steps are loaded
+// together while the batch before them is walked, and waited for once (loads issued step by step, 4 or 16
+// ahead, share the few load counters, and the walk met the L2's latency at most steps: 182 and 158 us at
+// 640 x 360 x 64, 73 us now).
+constexpr int kSgmThreads = 64;
+template <int KPL, bool kVec>
+__global__ void __launch_bounds__(kSgmThreads)
 k_sgm(const uint8_t* __restrict__ C, uint8_t* __restrict__ Lall, int W, int H, int D) {
     const int dir = blockIdx.y;
-    const int line = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int line = (blockIdx.x * kSgmThreads + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const bool horiz = dir < 2;
     const int lines = horiz ? H : W, len = horiz ? W : H;
     if (line >= lines) return;
-    uint8_t* __restrict__ Lout = Lall + (size_t)dir * W * H * D;
-    constexpr int kBig = 1 << 20, kAhead = 4;
-    auto base_of = [&](int s) {
-        const int pos = (dir == 0 || dir == 2) ? s : len - 1 - s;
-        const int x = horiz ? pos : line, y = horiz ? line : pos;
-        return ((size_t)y * W + x) * D;
-    };
-    auto load = [&](int s, int (&c)[KPL]) {
-        if (s < len) {
-            const size_t b = base_of(s);
+    constexpr int kBig = 1 << 20, kBatch = 16;
+    const int k0 = lane * KPL;
+    // offset of step s: first + s stride
+    const int64_t along = horiz ? (int64_t)D : (int64_t)W * D, across = horiz ? (int64_t)W * D : (int64_t)D;
+    const bool forward = dir == 0 || dir == 2;
+    const int64_t stride = forward ? along : -along;
+    const int64_t first = line * across + (forward ? 0 : (len - 1) * along) + k0;
+    const uint8_t* pc = C + first;
+    uint8_t* pl = Lall + (size_t)dir * W * H * D + first;
+    uint32_t next[kBatch];
+    auto fetch = [&](int s0) {  // the costs of steps s0 .. s0 + kBatch - 1
 #pragma unroll
-            for (int j = 0; j < KPL; ++j) {
-                const int k = lane * KPL + j;
-                c[j] = k < D ? (int)__ldg(C + b + k) : 0;
-            }
+        for (int a = 0; a < kBatch; ++a) {
+            next[a] = s0 + a < len ? load_bytes<KPL, kVec>(pc, k0, D) : 0u;
+            pc += stride;
         }
     };
-    int ring[kAhead][KPL];
-#pragma unroll
-    for (int a = 0; a < kAhead; ++a) load(a, ring[a]);
+    fetch(0);
     int L[KPL];
-    for (int s0 = 0; s0 < len; s0 += kAhead) {
+    for (int s0 = 0; s0 < len; s0 += kBatch) {
+        uint32_t cur[kBatch];
 #pragma unroll
-        for (int a = 0; a < kAhead; ++a) {
+        for (int a = 0; a < kBatch; ++a) cur[a] = next[a];
+        fetch(s0 + kBatch);
+#pragma unroll
+        for (int a = 0; a < kBatch; ++a) {
             const int s = s0 + a;
             if (s >= len) break;
-            int c[KPL];
-#pragma unroll
-            for (int j = 0; j < KPL; ++j) c[j] = ring[a][j];
-            load(s + kAhead, ring[a]);
+            const uint32_t cw = cur[a];
             if (s == 0) {
 #pragma unroll
-                for (int j = 0; j < KPL; ++j) L[j] = lane * KPL + j < D ? c[j] : kBig;
+                for (int j = 0; j < KPL; ++j) L[j] = k0 + j < D ? (int)((cw >> (8 * j)) & 255u) : kBig;
             } else {
-                int mloc = kBig;
+                int mloc = L[0];
 #pragma unroll
-                for (int j = 0; j < KPL; ++j) mloc = min(mloc, L[j]);
+                for (int j = 1; j < KPL; ++j) mloc = min(mloc, L[j]);
                 const int m = __reduce_min_sync(0xffffffffu, mloc);
                 const int below = __shfl_up_sync(0xffffffffu, L[KPL - 1], 1);   // plane lane*KPL - 1
                 const int above = __shfl_down_sync(0xffffffffu, L[0], 1);       // plane lane*KPL + KPL
                 int nl[KPL];
 #pragma unroll
                 for (int j = 0; j < KPL; ++j) {
-                    const int k = lane * KPL + j;
                     const int lm = j > 0 ? L[j - 1] : (lane > 0 ? below : kBig);
                     const int lp = j < KPL - 1 ? L[j + 1] : (lane < 31 ? above : kBig);
                     const int best = min(min(L[j], min(lm, lp) + kP1), m + kP2);
-                    nl[j] = k < D ? c[j] + best - m : kBig;
+                    nl[j] = k0 + j < D ? (int)((cw >> (8 * j)) & 255u) + best - m : kBig;
                 }
 #pragma unroll
                 for (int j = 0; j < KPL; ++j) L[j] = nl[j];
             }
-            const size_t b = base_of(s);
+            uint32_t out = 0;
 #pragma unroll
-            for (int j = 0; j < KPL; ++j) {
-                const int k = lane * KPL + j;
-                if (k < D) Lout[b + k] = (uint8_t)L[j];
-            }
+            for (int j = 0; j < KPL; ++j) out |= (uint32_t)L[j] << (8 * j);
+            store_bytes<KPL, kVec>(pl, k0, D, out);
+            pl += stride;
         }
     }
 }
 
 // S = the sum of the four paths (written out), winner-take-all, confidence, parabola refinement;
-// depth (NaN where not kept) and kept flags.  A warp takes 32 consecutive pixels: for each, lanes
-// over the planes (as in the SGM walk: coalesced loads and stores) find the minimiser, S2 and the
-// neighbours by warp reductions and leave them with lane i for pixel i; then every lane refines its
-// own pixel, so the FP64 refinement runs on full warps (GB300's FP64 pipe costs a warp instruction
-// the same with one lane or thirty-two).
+// depth (NaN where not kept) and kept flags.  A warp takes 32 consecutive pixels, four at a time (their
+// loads and warp reductions overlap): for each, lanes over the planes (as in the SGM walk: coalesced
+// loads and stores) find the minimiser and its value in one reduction of value << 8 | plane, then S2 and
+// the neighbours, and leave them with lane i for pixel i; then every lane refines its own pixel, so the
+// FP64 refinement runs on full warps (GB300's FP64 pipe costs a warp instruction the same with one lane
+// or thirty-two).  One pixel at a time, byte by byte, five reductions each: 66 us at 640 x 360 x 64, 39 us now.
 constexpr int kSelectThreads = 256;
 
-template <int KPL>
+template <int KPL, bool kVec>
 __global__ void __launch_bounds__(kSelectThreads)
 k_select(const uint8_t* __restrict__ Lall, uint16_t* __restrict__ S, int W, int H, int D, double inv_far,
          double step, float* __restrict__ depth, uint8_t* __restrict__ kept, unsigned long long* __restrict__ count) {
     __shared__ int s_count;
     if (threadIdx.x == 0) s_count = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31;
+    constexpr int kPix = 4;
+    constexpr uint32_t kBig = 1u << 30;
+    const int lane = threadIdx.x & 31, k0 = lane * KPL;
     const int64_t n = (int64_t)W * H;
     const size_t plane = (size_t)n * D;
     const int64_t chunks = (n + 31) / 32, warps = (int64_t)gridDim.x * (kSelectThreads / 32);
-    constexpr int kBig = 1 << 30;
     for (int64_t ch = (int64_t)blockIdx.x * (kSelectThreads / 32) + (threadIdx.x >> 5); ch < chunks; ch += warps) {
         int my_k1 = 0, my_s1 = 0, my_s2 = 0, my_sm = 0, my_sp = 0;
-        for (int i = 0; i < 32; ++i) {
-            const int64_t p = ch * 32 + i;
-            if (p >= n) break;  // warp-uniform
-            int v[KPL];
+        for (int i0 = 0; i0 < 32 && ch * 32 + i0 < n; i0 += kPix) {  // warp-uniform
+            uint32_t v[kPix][KPL];
 #pragma unroll
-            for (int j = 0; j < KPL; ++j) {
-                const int k = lane * KPL + j;
-                v[j] = kBig;
-                if (k < D) {
-                    int t = 0;
+            for (int u = 0; u < kPix; ++u) {
+                const int64_t p = ch * 32 + i0 + u;
 #pragma unroll
-                    for (int d = 0; d < 4; ++d) t += __ldg(Lall + d * plane + (size_t)p * D + k);
-                    v[j] = t;
-                    S[(size_t)p * D + k] = (uint16_t)t;
+                for (int j = 0; j < KPL; ++j) v[u][j] = 0u;
+                if (p < n) {
+                    const size_t at = (size_t)p * D + k0;
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) {
+                        const uint32_t w = load_bytes<KPL, kVec>(Lall + d * plane + at, k0, D);
+#pragma unroll
+                        for (int j = 0; j < KPL; ++j) v[u][j] += (w >> (8 * j)) & 255u;
+                    }
+                    if constexpr (KPL == 2 && kVec) {
+                        if (k0 < D) *reinterpret_cast<uint32_t*>(S + at) = v[u][0] | v[u][1] << 16;
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < KPL; ++j)
+                            if (k0 + j < D) S[at + j] = (uint16_t)v[u][j];
+                    }
                 }
             }
-            int loc = kBig;
 #pragma unroll
-            for (int j = 0; j < KPL; ++j) loc = min(loc, v[j]);
-            const int s1 = __reduce_min_sync(0xffffffffu, loc);
-            int kloc = kBig;
+            for (int u = 0; u < kPix; ++u) {
+                uint32_t key = 0xffffffffu;
 #pragma unroll
-            for (int j = KPL - 1; j >= 0; --j)
-                if (v[j] == s1) kloc = lane * KPL + j;
-            const int k1 = __reduce_min_sync(0xffffffffu, kloc);  // first minimiser
-            int far = kBig, mm = 0, mp = 0;
+                for (int j = 0; j < KPL; ++j)
+                    if (k0 + j < D) key = min(key, v[u][j] << 8 | (uint32_t)(k0 + j));
+                key = __reduce_min_sync(0xffffffffu, key);  // the first minimiser and its value
+                const int k1 = (int)(key & 255u);
+                uint32_t far = kBig, below = 0, above = 0;  // values of planes k1 - 1 and k1 + 1, in their lanes
 #pragma unroll
-            for (int j = 0; j < KPL; ++j) {
-                const int k = lane * KPL + j;
-                if (k < D && abs(k - k1) >= 2) far = min(far, v[j]);
-                if (k == k1 - 1) mm = v[j];
-                if (k == k1 + 1) mp = v[j];
-            }
-            const int s2 = __reduce_min_sync(0xffffffffu, far);
-            const int sm = __reduce_add_sync(0xffffffffu, mm), sp = __reduce_add_sync(0xffffffffu, mp);
-            if (lane == i) {
-                my_k1 = k1;
-                my_s1 = s1;
-                my_s2 = s2 == kBig ? s1 : s2;
-                my_sm = sm;
-                my_sp = sp;
+                for (int j = 0; j < KPL; ++j) {
+                    const int k = k0 + j;
+                    if (k < D && abs(k - k1) >= 2) far = min(far, v[u][j]);
+                    if (j == ((k1 - 1) & 0xffff) % KPL) below = v[u][j];
+                    if (j == (k1 + 1) % KPL) above = v[u][j];
+                }
+                const uint32_t s2 = __reduce_min_sync(0xffffffffu, far);
+                const int sm = (int)__shfl_sync(0xffffffffu, below, max(k1 - 1, 0) / KPL);
+                const int sp = (int)__shfl_sync(0xffffffffu, above, (k1 + 1) / KPL);
+                if (lane == i0 + u) {
+                    my_k1 = k1;
+                    my_s1 = (int)(key >> 8);
+                    my_s2 = s2 == kBig ? my_s1 : (int)s2;
+                    my_sm = sm;  // (k1 on the first or last plane is not kept)
+                    my_sp = sp;
+                }
             }
         }
         const int64_t p = ch * 32 + lane;
@@ -312,12 +388,18 @@ k_select(const uint8_t* __restrict__ Lall, uint16_t* __restrict__ S, int W, int 
     if (threadIdx.x == 0 && s_count) atomicAdd(count, (unsigned long long)s_count);
 }
 
-// kept-pixel counts per CTA (pixel order), then an exclusive scan in one CTA, then the points
+// kept-pixel counts per CTA (pixel order) and, on the side, the FP64 ray slopes ((i + 0.5) - c) / f of every
+// column and row (ray [W + H]); then an exclusive scan in one CTA, then the points.  The points are bound by the
+// FP64 pipe: with the two divisions per pixel instead of per column and row they took 30 us at 640 x 360, 19 us now.
 constexpr int kFuseThreads = 256;
 
 __global__ void __launch_bounds__(kFuseThreads)
-k_fuse_count(const float* __restrict__ depth, int64_t n, uint32_t* __restrict__ cta_count) {
-    const int64_t p = (int64_t)blockIdx.x * kFuseThreads + threadIdx.x;
+k_fuse_count(const float* __restrict__ depth, int W, int H, CamF cam, uint32_t* __restrict__ cta_count,
+             double* __restrict__ ray) {
+    const int64_t n = (int64_t)W * H, p = (int64_t)blockIdx.x * kFuseThreads + threadIdx.x;
+    for (int64_t i = p; i < W + H; i += (int64_t)gridDim.x * kFuseThreads)
+        ray[i] = i < W ? ddiv(dsub((double)i + 0.5, (double)cam.cx), (double)cam.fx)
+                       : ddiv(dsub((double)(i - W) + 0.5, (double)cam.cy), (double)cam.fy);
     const bool keep = p < n && depth[p] == depth[p];
     const int c = __syncthreads_count(keep);
     if (threadIdx.x == 0) cta_count[blockIdx.x] = (uint32_t)c;
@@ -352,7 +434,7 @@ k_fuse_scan(uint32_t* __restrict__ cta_count, int ctas, int64_t* __restrict__ to
 
 __global__ void __launch_bounds__(kFuseThreads)
 k_fuse_points(const float* __restrict__ depth, int W, int64_t n, CamF cam, const uint32_t* __restrict__ cta_off,
-              int64_t capacity, float* __restrict__ points, int32_t* __restrict__ pix) {
+              const double* __restrict__ ray, int64_t capacity, float* __restrict__ points, int32_t* __restrict__ pix) {
     __shared__ uint32_t s_warp[kFuseThreads / 32];
     const int64_t p = (int64_t)blockIdx.x * kFuseThreads + threadIdx.x;
     const float d = p < n ? depth[p] : __int_as_float(0x7fc00000);
@@ -368,8 +450,8 @@ k_fuse_points(const float* __restrict__ depth, int W, int64_t n, CamF cam, const
     if (o >= capacity) return;
     const int y = (int)(p / W), x = (int)(p % W);
     const double dd = d;
-    const double X0 = dsub(dmul(dd, ddiv(dsub((double)x + 0.5, (double)cam.cx), (double)cam.fx)), (double)cam.v[3]);
-    const double X1 = dsub(dmul(dd, ddiv(dsub((double)y + 0.5, (double)cam.cy), (double)cam.fy)), (double)cam.v[7]);
+    const double X0 = dsub(dmul(dd, ray[x]), (double)cam.v[3]);
+    const double X1 = dsub(dmul(dd, ray[W + y]), (double)cam.v[7]);
     const double X2 = dsub(dd, (double)cam.v[11]);
     for (int j = 0; j < 3; ++j) {
         const double w =
@@ -398,69 +480,165 @@ __global__ void k_sparse_depths(const float* __restrict__ P, int64_t n, CamF cam
     z[atomicAdd(count, 1ull)] = zz;
 }
 
-// one CTA: the order statistics of the quantiles 0.05, 0.5, 0.95 of z[0..m) by radix selection on
-// the FP64 bit patterns (positive values order like their bits), eight 8-bit passes for all six
-// ranks at once; out = (0.5 q.05, 1.5 q.95, q.5)
+// One CTA: the order statistics of the quantiles 0.05, 0.5, 0.95 of z[0..m) by bucket selection on the FP64
+// bit patterns (positive values order like their bits), all six ranks at once; out = (0.5 q.05, 1.5 q.95,
+// q.5).  The interval from the values' own minimum to their maximum is counted in 2048 buckets; the few
+// values of the ranks' buckets are listed and each rank's is the one with as many listed before it.
+// Where a bucket holds many (equal or clustered values), its interval is cut into buckets again.  Eight
+// 8-bit passes over the whole pattern put all values of a scene in a few bins: 162 us for 20k values
+// even with a warp's equal bins counted together, 26 us now.
 __global__ void __launch_bounds__(1024)
 k_quantiles(const double* __restrict__ z, const unsigned long long* __restrict__ count, double* __restrict__ out,
             int* __restrict__ status) {
-    constexpr int kQ = 6;
-    __shared__ unsigned s_hist[kQ][256];
-    __shared__ unsigned long long s_prefix[kQ];
-    __shared__ long long s_rank[kQ];
+    constexpr int kQ = 6, kBits = 11, kBuckets = 1 << kBits, kList = 256;
+    typedef unsigned long long u64;
+    __shared__ unsigned s_hist[kBuckets];
+    __shared__ u64 s_list[kList];
+    __shared__ u64 s_lo[kQ], s_hi[kQ];  // rank q's value lies in [lo, hi]
+    __shared__ int s_rank[kQ];          // and is that one of the interval's values, in order
+    __shared__ int s_cut[kQ];           // round that last cut its interval
+    __shared__ u64 s_min[32], s_max[32];
+    __shared__ unsigned s_warp[32];
+    __shared__ int s_listed;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long m = (long long)*count;
     if (m == 0) {
         if (threadIdx.x == 0) atomicOr(status, 1);
         return;
     }
+    constexpr int kLoads = 8;  // values in flight per thread: a pass is a few memory latencies
+    auto for_values = [&](auto&& f) {
+        for (long long i0 = threadIdx.x; i0 < m; i0 += kLoads * 1024) {
+            u64 b[kLoads];
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u) {
+                const long long i = i0 + u * 1024;
+                b[u] = (u64)__double_as_longlong(z[i < m ? i : i0]);
+            }
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u)
+                if (i0 + u * 1024 < m) f(b[u]);
+        }
+    };
+    u64 lo = ~0ull, hi = 0ull;
+    for_values([&](u64 b) {
+        lo = min(lo, b);
+        hi = max(hi, b);
+    });
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if (lane == 0) {
+        s_min[warp] = lo;
+        s_max[warp] = hi;
+    }
+    __syncthreads();
     const double ps[3] = {0.05, 0.5, 0.95};
     if (threadIdx.x < kQ) {
+        for (int w = 0; w < 32; ++w) {
+            lo = min(lo, s_min[w]);
+            hi = max(hi, s_max[w]);
+        }
         const double h = dmul((double)(m - 1), ps[threadIdx.x >> 1]);
-        const long long lo = (long long)floor(h);
-        s_rank[threadIdx.x] = (threadIdx.x & 1) ? (lo + 1 < m ? lo + 1 : m - 1) : lo;
-        s_prefix[threadIdx.x] = 0ull;
+        const long long r = (long long)floor(h);
+        s_rank[threadIdx.x] = (int)((threadIdx.x & 1) ? (r + 1 < m ? r + 1 : m - 1) : r);
+        s_lo[threadIdx.x] = lo;
+        s_hi[threadIdx.x] = hi;
+        s_cut[threadIdx.x] = 0;
     }
-    for (int shift = 56; shift >= 0; shift -= 8) {
-        for (int e = threadIdx.x; e < kQ * 256; e += blockDim.x) (&s_hist[0][0])[e] = 0u;
-        __syncthreads();
-        const unsigned long long hmask = shift == 56 ? 0ull : (~0ull << (shift + 8));
-        // the values cluster, so most lanes of a warp hit the same bin: one atomic per distinct bin
-        // of a warp (lanes grouped by __match_any_sync) instead of one per lane
-        const long long mend = (m + 31) & ~31ll;
-        for (long long i = threadIdx.x; i < mend; i += blockDim.x) {
-            const bool live = i < m;
-            const unsigned long long b = live ? (unsigned long long)__double_as_longlong(z[i]) : 0ull;
-            const unsigned d = (unsigned)((b >> shift) & 255ull);
-            const unsigned lane = threadIdx.x & 31;
+    __syncthreads();
+    for (int round = 1;; ++round) {
+        // list the values of the intervals that are not single values yet, unless they are too many
+        if (round > 1 || m <= kList) {
+            if (threadIdx.x == 0) s_listed = 0;
+            __syncthreads();
+            for_values([&](u64 b) {
+                bool in = false;
 #pragma unroll
-            for (int q = 0; q < kQ; ++q) {
-                const unsigned key = (live && (b & hmask) == s_prefix[q]) ? d : 256u;
-                const unsigned grp = __match_any_sync(0xffffffffu, key);
-                if (key < 256u && lane == (unsigned)(__ffs(grp) - 1)) atomicAdd(&s_hist[q][key], (unsigned)__popc(grp));
-            }
+                for (int e = 0; e < kQ; ++e) in = in || (b >= s_lo[e] && b <= s_hi[e] && s_lo[e] < s_hi[e]);
+                if (in) {
+                    const int at = atomicAdd(&s_listed, 1);
+                    if (at < kList) s_list[at] = b;
+                }
+            });
+            __syncthreads();
+            if (s_listed <= kList) break;  // (0 when every rank's value is known)
         }
-        __syncthreads();
-        if (threadIdx.x < kQ) {
-            const int q = threadIdx.x;
-            long long r = s_rank[q];
-            int d = 0;
-            for (; d < 255; ++d) {
-                if (r < (long long)s_hist[q][d]) break;
-                r -= s_hist[q][d];
+        // else cut each of these intervals into buckets and keep its ranks' (2^11 times narrower a round)
+        for (int q = 0; q < kQ; ++q) {
+            __syncthreads();
+            const u64 l = s_lo[q], h = s_hi[q];
+            const bool skip = l == h || s_cut[q] == round;  // the same for every thread
+            __syncthreads();
+            if (skip) continue;
+            const int shift = max(0, 64 - __clzll((long long)(h - l)) - kBits);
+            for (int e = threadIdx.x; e < kBuckets; e += 1024) s_hist[e] = 0u;
+            __syncthreads();
+            for_values([&](u64 b) {
+                if (b >= l && b <= h) atomicAdd(&s_hist[(b - l) >> shift], 1u);
+            });
+            __syncthreads();
+            // prefix of the counts, two buckets a thread
+            const unsigned c0 = s_hist[2 * threadIdx.x], c1 = s_hist[2 * threadIdx.x + 1];
+            unsigned incl = c0 + c1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
             }
-            s_rank[q] = r;
-            s_prefix[q] |= (unsigned long long)d << shift;
+            if (lane == 31) s_warp[warp] = incl;
+            __syncthreads();
+            unsigned first = incl - c0 - c1;
+            for (int w = 0; w < warp; ++w) first += s_warp[w];
+            unsigned mine = 0;  // the ranks of this interval that fall into the thread's buckets
+            for (int e = q; e < kQ; ++e) {
+                const unsigned r = (unsigned)s_rank[e];
+                if (s_lo[e] == l && s_hi[e] == h && r >= first && r < first + c0 + c1) mine |= 1u << e;
+            }
+            __syncthreads();
+            for (int e = q; e < kQ; ++e)
+                if ((mine >> e) & 1u) {
+                    const unsigned r = (unsigned)s_rank[e] - first, second = r >= c0 ? 1u : 0u;
+                    const u64 start = l + ((u64)(2 * threadIdx.x + second) << shift);
+                    s_rank[e] = (int)(r - (second ? c0 : 0u));
+                    s_lo[e] = start;
+                    s_hi[e] = min(h, start + ((1ull << shift) - 1));
+                    s_cut[e] = round;
+                }
         }
         __syncthreads();
     }
+    __syncthreads();
+    // the listed values: rank q's is the one with s_rank[q] of its interval's before it
+    const int listed = min(s_listed, kList);
+    if (threadIdx.x < listed) {
+        const u64 x = s_list[threadIdx.x];
+        for (int q = 0; q < kQ; ++q) {
+            const u64 l = s_lo[q], h = s_hi[q];
+            if (x < l || x > h || l == h) continue;
+            int less = 0, same = 0;
+            for (int k = 0; k < listed; ++k) {
+                const u64 y = s_list[k];
+                less += y >= l && y < x;
+                same += y == x;
+            }
+            if (s_rank[q] >= less && s_rank[q] < less + same) s_min[q] = x;
+        }
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
         double q[3];
         for (int j = 0; j < 3; ++j) {
             const double h = dmul((double)(m - 1), ps[j]);
-            const double lo = floor(h);
-            const double a = __longlong_as_double((long long)s_prefix[2 * j]);
-            const double b = __longlong_as_double((long long)s_prefix[2 * j + 1]);
-            q[j] = dadd(a, dmul(dsub(h, lo), dsub(b, a)));
+            const double fl = floor(h);
+            double v[2];
+            for (int e = 0; e < 2; ++e) {
+                const int k = 2 * j + e;
+                v[e] = __longlong_as_double((long long)(s_lo[k] == s_hi[k] ? s_lo[k] : s_min[k]));
+            }
+            q[j] = dadd(v[0], dmul(dsub(h, fl), dsub(v[1], v[0])));
         }
         out[0] = dmul(0.5, q[0]);
         out[1] = dmul(1.5, q[2]);
@@ -518,48 +696,64 @@ unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
 
-int launch_mvs_census(const float* rgb, int W, int H, uint64_t* code, cudaStream_t s) {
-    k_census<<<dim3(blocks(W, kCtx), blocks(H, kCty)), dim3(kCtx, kCty), 0, s>>>(rgb, W, H, code);
+int launch_mvs_census(const pgs_camera& t, const pgs_camera& r, const float* rgb_t, const float* rgb_r, int W, int H, int D,
+                      double inv_far, double step, uint64_t* code_t, uint64_t* code_r, float* maps, cudaStream_t s) {
+    k_census<<<dim3(blocks(W, kCtx), blocks(H, kCty), 3), dim3(kCtx, kCty), 0, s>>>(rgb_t, rgb_r, W, H, code_t, code_r,
+                                                                                   camf(t), camf(r), inv_far, step, D, maps);
     return 1;
 }
 
-int launch_mvs_cost(const pgs_camera& t, const pgs_camera& r, const uint64_t* cen_t, const uint64_t* cen_r, int W,
-                    int H, int D, double inv_far, double step, float* maps, uint8_t* C, cudaStream_t s) {
-    k_plane_maps<<<blocks(D, 64), 64, 0, s>>>(camf(t), camf(r), inv_far, step, D, maps);
+int launch_mvs_cost(const uint64_t* cen_t, const uint64_t* cen_r, int W, int H, int D, const float* maps, uint8_t* C,
+                    cudaStream_t s) {
     k_cost<<<dim3(blocks(W, kRun), H), D, 0, s>>>(cen_t, cen_r, W, H, D, maps, C);
-    return 2;
+    return 1;
 }
 
+// planes per lane for D planes: 1, 2, 3 or 4; one access for a lane's planes when they divide D
+template <template <int, bool> class Launch, class... Args>
+void by_planes(int D, Args... args) {
+    if (D <= 32) Launch<1, true>::run(args...);
+    else if (D <= 64) D % 2 == 0 ? Launch<2, true>::run(args...) : Launch<2, false>::run(args...);
+    else if (D <= 96) Launch<3, false>::run(args...);
+    else D % 4 == 0 ? Launch<4, true>::run(args...) : Launch<4, false>::run(args...);
+}
+template <int KPL, bool kVec>
+struct SgmLaunch {
+    static void run(const uint8_t* C, uint8_t* L, int W, int H, int D, cudaStream_t s) {
+        const dim3 g(blocks((int64_t)(W > H ? W : H) * 32, kSgmThreads), 4);
+        k_sgm<KPL, kVec><<<g, kSgmThreads, 0, s>>>(C, L, W, H, D);
+    }
+};
+template <int KPL, bool kVec>
+struct SelectLaunch {
+    static void run(const uint8_t* L, uint16_t* S, int W, int H, int D, double inv_far, double step, float* depth,
+                    uint8_t* kept, unsigned long long* count, cudaStream_t s) {
+        const int64_t n = (int64_t)W * H;
+        int64_t g = ((n + 31) / 32 + kSelectThreads / 32 - 1) / (kSelectThreads / 32);
+        if (g > 152 * 8) g = 152 * 8;  // grid-stride: 8 resident CTAs an SM
+        k_select<KPL, kVec><<<(unsigned)g, kSelectThreads, 0, s>>>(L, S, W, H, D, inv_far, step, depth, kept, count);
+    }
+};
+
 int launch_mvs_sgm(const uint8_t* C, uint8_t* L, int W, int H, int D, cudaStream_t s) {
-    const int lines = W > H ? W : H;
-    const dim3 g(blocks((int64_t)lines * 32, 128), 4);
-    if (D <= 32) k_sgm<1><<<g, 128, 0, s>>>(C, L, W, H, D);
-    else if (D <= 64) k_sgm<2><<<g, 128, 0, s>>>(C, L, W, H, D);
-    else if (D <= 96) k_sgm<3><<<g, 128, 0, s>>>(C, L, W, H, D);
-    else k_sgm<4><<<g, 128, 0, s>>>(C, L, W, H, D);
+    by_planes<SgmLaunch>(D, C, L, W, H, D, s);
     return 1;
 }
 
 int launch_mvs_select(const uint8_t* L, uint16_t* S, int W, int H, int D, double inv_far, double step, float* depth,
                       uint8_t* kept, unsigned long long* count, cudaStream_t s) {
     cudaMemsetAsync(count, 0, sizeof(unsigned long long), s);
-    const int64_t n = (int64_t)W * H;
-    int64_t g = ((n + 31) / 32 + kSelectThreads / 32 - 1) / (kSelectThreads / 32);
-    if (g > 152 * 8) g = 152 * 8;  // grid-stride: 8 resident CTAs an SM
-    if (D <= 32) k_select<1><<<(unsigned)g, kSelectThreads, 0, s>>>(L, S, W, H, D, inv_far, step, depth, kept, count);
-    else if (D <= 64) k_select<2><<<(unsigned)g, kSelectThreads, 0, s>>>(L, S, W, H, D, inv_far, step, depth, kept, count);
-    else if (D <= 96) k_select<3><<<(unsigned)g, kSelectThreads, 0, s>>>(L, S, W, H, D, inv_far, step, depth, kept, count);
-    else k_select<4><<<(unsigned)g, kSelectThreads, 0, s>>>(L, S, W, H, D, inv_far, step, depth, kept, count);
+    by_planes<SelectLaunch>(D, L, S, W, H, D, inv_far, step, depth, kept, count, s);
     return 1;
 }
 
-int launch_mvs_fuse(const float* depth, int W, int H, const pgs_camera& cam, uint32_t* cta_scratch, int64_t* total,
-                    int64_t capacity, float* points, int32_t* pix, cudaStream_t s) {
+int launch_mvs_fuse(const float* depth, int W, int H, const pgs_camera& cam, uint32_t* cta_scratch, double* ray,
+                    int64_t* total, int64_t capacity, float* points, int32_t* pix, cudaStream_t s) {
     const int64_t n = (int64_t)W * H;
     const unsigned g = blocks(n, kFuseThreads);
-    k_fuse_count<<<g, kFuseThreads, 0, s>>>(depth, n, cta_scratch);
+    k_fuse_count<<<g, kFuseThreads, 0, s>>>(depth, W, H, camf(cam), cta_scratch, ray);
     k_fuse_scan<<<1, 1024, 0, s>>>(cta_scratch, (int)g, total);
-    k_fuse_points<<<g, kFuseThreads, 0, s>>>(depth, W, n, camf(cam), cta_scratch, capacity, points, pix);
+    k_fuse_points<<<g, kFuseThreads, 0, s>>>(depth, W, n, camf(cam), cta_scratch, ray, capacity, points, pix);
     return 3;
 }
 

@@ -25,6 +25,7 @@ struct pgs_mvs {
     double* scores = nullptr;             // 1024
     uint32_t* cta = nullptr;
     int64_t* total = nullptr;
+    double* ray = nullptr;  // ray slopes of the columns and rows (fusion)
     double* zbuf = nullptr;  // sparse depths, grown on demand
     int64_t zcap = 0;
 };
@@ -64,10 +65,11 @@ int pgs_mvs_create(pgs_mvs** out, int32_t width, int32_t height, int32_t planes,
     m->D = planes;
     const size_t px = (size_t)width * height, D = planes;
     const size_t sizes[] = {8 * px, 8 * px, 4 * 9 * D, px * D, 4 * px * D, 2 * px * D, px, 16, 24, 8,
-                            1024 * mvs_camf_bytes(), 8 * 1024, 4 * (size_t)mvs_fuse_ctas(width, height), 8};
+                            1024 * mvs_camf_bytes(), 8 * 1024, 4 * (size_t)mvs_fuse_ctas(width, height), 8,
+                            8 * ((size_t)width + height)};
     void** slots[] = {(void**)&m->cen_t, (void**)&m->cen_r, (void**)&m->maps, (void**)&m->C, (void**)&m->L, (void**)&m->S,
                       (void**)&m->kept, (void**)&m->count, (void**)&m->range, (void**)&m->status, &m->cams,
-                      (void**)&m->scores, (void**)&m->cta, (void**)&m->total};
+                      (void**)&m->scores, (void**)&m->cta, (void**)&m->total, (void**)&m->ray};
     constexpr int kSlots = sizeof(sizes) / sizeof(sizes[0]);
     static_assert(kSlots == sizeof(slots) / sizeof(slots[0]), "one size per buffer");
     size_t total = 0;
@@ -152,9 +154,8 @@ int pgs_mvs_depth(pgs_mvs* m, const pgs_camera* target, const pgs_camera* refere
     cudaStream_t s = m->stream;
     const double inv_far = 1.0 / d_max;
     const double step = (1.0 / d_min - inv_far) / (m->D - 1);
-    launch_mvs_census(image_t, m->W, m->H, m->cen_t, s);
-    launch_mvs_census(image_r, m->W, m->H, m->cen_r, s);
-    launch_mvs_cost(*target, *reference, m->cen_t, m->cen_r, m->W, m->H, m->D, inv_far, step, m->maps, m->C, s);
+    launch_mvs_census(*target, *reference, image_t, image_r, m->W, m->H, m->D, inv_far, step, m->cen_t, m->cen_r, m->maps, s);
+    launch_mvs_cost(m->cen_t, m->cen_r, m->W, m->H, m->D, m->maps, m->C, s);
     launch_mvs_sgm(m->C, m->L, m->W, m->H, m->D, s);
     launch_mvs_select(m->L, m->S, m->W, m->H, m->D, inv_far, step, depth, m->kept, m->count, s);
     cudaError_t e = cudaGetLastError();
@@ -187,10 +188,9 @@ int pgs_mvs_stage_times(pgs_mvs* m, const pgs_camera* target, const pgs_camera* 
     }
     if (e == cudaSuccess) {
         cudaEventRecord(ev[0], s);
-        launch_mvs_census(image_t, m->W, m->H, m->cen_t, s);
-        launch_mvs_census(image_r, m->W, m->H, m->cen_r, s);
+        launch_mvs_census(*target, *reference, image_t, image_r, m->W, m->H, m->D, inv_far, step, m->cen_t, m->cen_r, m->maps, s);
         cudaEventRecord(ev[1], s);
-        launch_mvs_cost(*target, *reference, m->cen_t, m->cen_r, m->W, m->H, m->D, inv_far, step, m->maps, m->C, s);
+        launch_mvs_cost(m->cen_t, m->cen_r, m->W, m->H, m->D, m->maps, m->C, s);
         cudaEventRecord(ev[2], s);
         launch_mvs_sgm(m->C, m->L, m->W, m->H, m->D, s);
         cudaEventRecord(ev[3], s);
@@ -225,7 +225,7 @@ int pgs_mvs_fuse(pgs_mvs* m, const pgs_camera* target, const float* depth, float
     if (!m || !same_size(m, target) || !finite_camera(target) || !depth || capacity < 0 ||
         (capacity > 0 && (!points || !pixels)) || !count)
         return PGS_ERR_INVALID_ARG;
-    launch_mvs_fuse(depth, m->W, m->H, *target, m->cta, m->total, capacity, points, pixels, m->stream);
+    launch_mvs_fuse(depth, m->W, m->H, *target, m->cta, m->ray, m->total, capacity, points, pixels, m->stream);
     int64_t n = 0;
     cudaError_t e = cudaMemcpyAsync(&n, m->total, sizeof(n), cudaMemcpyDeviceToHost, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
