@@ -28,6 +28,7 @@
 #include <cstdlib>
 #include <type_traits>
 
+#include "f32x2.cuh"
 #include "pgs_internal.cuh"
 
 namespace pgs {
@@ -509,41 +510,6 @@ __device__ __forceinline__ void bwd_tile_scalar(const TileJob& J, int64_t n, con
 // bit-identical to the one-pixel tiles; per pixel the work is branch-free (a pixel that
 // does not composite an entry contributes alpha = 0, which leaves T, C and the colour behind
 // unchanged), and the pair shares one branch.
-struct F2 {
-    unsigned long long r;
-};
-__device__ __forceinline__ F2 f2(float a, float b) {
-    F2 o;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(o.r) : "f"(a), "f"(b));
-    return o;
-}
-__device__ __forceinline__ F2 f2(float a) { return f2(a, a); }
-__device__ __forceinline__ float2 un(F2 a) {
-    float2 o;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(a.r));
-    return o;
-}
-__device__ __forceinline__ F2 add2(F2 a, F2 b) {
-    F2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d.r) : "l"(a.r), "l"(b.r));
-    return d;
-}
-__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
-    F2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d.r) : "l"(a.r), "l"(b.r));
-    return d;
-}
-__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
-    F2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d.r) : "l"(a.r), "l"(b.r));
-    return d;
-}
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
-    F2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.r) : "l"(a.r), "l"(b.r), "l"(c.r));
-    return d;
-}
-
 // alpha of the pixel pair (dy, dy + 1) below one entry: the packed form of entry_alpha
 __device__ __forceinline__ void pair_alpha(F2 dy, F2 DX, F2 ADX2, F2 S2Y, F2 S2Z, F2 O, float2& G,
                                            float2& og, float2& alpha) {

@@ -2,9 +2,9 @@
 // accumulation on the tensor cores (mma.sync m16n8k16, bf16 x bf16 -> f32), operands staged in
 // shared memory and loaded with ldmatrix (transposed where a product needs the transpose).
 //
-// At K = 16 / 64 and N = 8 / 64 each layer is a handful of 16x8x16 products per 16 points; the
-// kernels keep every activation of a 64-point slice in shared memory, so a training step reads
-// the features and targets once and writes only the loss and the weight gradients.
+// At K = 16 / 64 and N = 8 / 64 each layer is a handful of 16x8x16 products per 16 points, and the 128 GELUs
+// a point take the time.  Both kernels carry a warp's 16 points through the layers in registers;
+// a training step reads the features and targets once and writes only the loss and the weight gradients.
 //
 // Training kernel, per CTA slice of 64 points (4 warps x 16):
 //   forward  Z1 = X W1^T + b1, H1 = gelu(Z1), Z2 = H1 W2^T + b2, H2 = gelu(Z2), Y = H2 W3^T + b3
@@ -16,6 +16,7 @@
 // BF16 rounding points: X, weights, H1, H2 and the gradients fed to products (dY, dZ2, dZ1).
 #include <cuda_bf16.h>
 
+#include "f32x2.cuh"
 #include "pgs_internal.cuh"
 
 namespace pgs {
@@ -41,10 +42,6 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t r[4], const void* p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)));
 }
-__device__ __forceinline__ void ldsm_x2(uint32_t r[2], const void* p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n"
-                 : "=r"(r[0]), "=r"(r[1]) : "r"(smem_addr(p)));
-}
 __device__ __forceinline__ void ldsm_x2_t(uint32_t r[2], const void* p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
                  : "=r"(r[0]), "=r"(r[1]) : "r"(smem_addr(p)));
@@ -56,405 +53,425 @@ __device__ __forceinline__ void mma(float c[4], const uint32_t a[4], const uint3
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// A fragment (16 x 16) of a row-major bf16 matrix at (r0, c0)
-__device__ __forceinline__ void frag_a(uint32_t a[4], const __nv_bfloat16* S, int ld, int r0, int c0) {
-    const int l = threadIdx.x & 31, i = l >> 3;
-    ldsm_x4(a, S + (size_t)(r0 + (i & 1) * 8 + (l & 7)) * ld + c0 + (i >> 1) * 8);
+__device__ __forceinline__ void mma_k8(float c[4], const uint32_t a[2], uint32_t b) {
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 "
+                 "{%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};\n"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(b));
 }
+
 // A fragment of the transpose: A[m][k] = S[k][m], block rows (data) k0.., cols m0..
 __device__ __forceinline__ void frag_a_t(uint32_t a[4], const __nv_bfloat16* S, int ld, int k0, int m0) {
     const int l = threadIdx.x & 31, i = l >> 3;
     ldsm_x4_t(a, S + (size_t)(k0 + (i >> 1) * 8 + (l & 7)) * ld + m0 + (i & 1) * 8);
 }
-// B fragment (16 x 8) with B[k][n] = W[n][k], W row-major [n][k]
-__device__ __forceinline__ void frag_b(uint32_t b[2], const __nv_bfloat16* W, int ld, int n0, int k0) {
-    const int l = threadIdx.x & 31;
-    ldsm_x2(b, W + (size_t)(n0 + (l & 7)) * ld + k0 + ((l >> 3) & 1) * 8);
-}
-// B fragment with B[k][n] = S[k][n], S row-major [k][n]
-__device__ __forceinline__ void frag_b_t(uint32_t b[2], const __nv_bfloat16* S, int ld, int k0, int n0) {
-    const int l = threadIdx.x & 31;
-    ldsm_x2_t(b, S + (size_t)(k0 + ((l >> 3) & 1) * 8 + (l & 7)) * ld + n0);
-}
-
 // 1 + erf(x) by the rational approximation 7.1.26 of Abramowitz & Stegun (Handbook of
 // Mathematical Functions, 1964): for x >= 0, erf(x) = 1 - (a1 s + a2 s^2 + ... + a5 s^5) e^{-x^2}
 // with s = 1 / (1 + p x) and |error| <= 1.5e-7, far below the BF16 rounding of the activations.
 // Evaluated as q = polynomial * e^{-x^2}, 1 + erf(x) = 2 - q for x >= 0 and q for x < 0 (the
 // odd symmetry), so the left tail keeps its relative accuracy instead of cancelling.
-__device__ __forceinline__ float one_plus_erf(float x) {
-    const float ax = fabsf(x);
-    const float s = __fdividef(1.0f, fmaf(0.3275911f, ax, 1.0f));
-    float poly = fmaf(1.061405429f, s, -1.453152027f);
-    poly = fmaf(poly, s, 1.421413741f);
-    poly = fmaf(poly, s, -0.284496736f);
-    poly = fmaf(poly, s, 0.254829592f);
-    const float q = poly * s * __expf(-ax * ax);
-    return x >= 0.0f ? 2.0f - q : q;
+//
+// Two arguments at a time, in the halves: returns Phi of both, Phi(z) = (1 + erf(z / sqrt 2)) / 2 (the
+// factor 1/2 is exact in the coefficients), and e = e^{-z^2 / 2}.
+__device__ __forceinline__ F2 phi2(F2 z, F2& e) {
+    const F2 x = mul2(z, f2(0.70710678118654752f));
+    const float2 xv = un(x);
+    // ex2 and rcp with flushed subnormals: the arguments of rcp are at least 1, and e^{-x^2} below 2^-126
+    // changes no activation's sum
+    const float2 w = un(mul2(mul2(x, x), f2(-1.4426950408889634f)));
+    F2 s;
+    {
+        float a, b;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(fmaf(0.3275911f, fabsf(xv.x), 1.0f)));
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(fmaf(0.3275911f, fabsf(xv.y), 1.0f)));
+        s = f2(a, b);
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(w.x));
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"(w.y));
+        e = f2(a, b);
+    }
+    F2 poly = fma2(f2(0.5f * 1.061405429f), s, f2(0.5f * -1.453152027f));
+    poly = fma2(poly, s, f2(0.5f * 1.421413741f));
+    poly = fma2(poly, s, f2(0.5f * -0.284496736f));
+    poly = fma2(poly, s, f2(0.5f * 0.254829592f));
+    const F2 ps = mul2(poly, s);
+    const float2 q = un(mul2(ps, e));
+    return f2(xv.x >= 0.0f ? __fsub_rn(1.0f, q.x) : q.x, xv.y >= 0.0f ? __fsub_rn(1.0f, q.y) : q.y);
 }
-// GELU in the erf form, z Phi(z), and its derivative Phi(z) + z phi(z)
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * one_plus_erf(z * 0.70710678118654752f); }
-__device__ __forceinline__ float gelu_d(float z) {
-    return 0.5f * one_plus_erf(z * 0.70710678118654752f) + z * __expf(-0.5f * z * z) * 0.3989422804014327f;
+// GELU in the erf form, z Phi(z), and with its derivative d = Phi(z) + z phi(z)
+__device__ __forceinline__ F2 gelu2(F2 z) {
+    F2 e;
+    return mul2(z, phi2(z, e));
+}
+__device__ __forceinline__ F2 gelu2(F2 z, F2& d) {
+    F2 e;
+    const F2 p = phi2(z, e);
+    d = fma2(mul2(z, e), f2(0.3989422804014327f), p);
+    return mul2(z, p);
 }
 
-struct Smem {
-    __nv_bfloat16 W1[kHid * LD16], W2[kHid * LD64], W3[16 * LD64];  // W3 rows 8..15 zero
-    __nv_bfloat16 X[kRows * LD16], H1[kRows * LD64], H2[kRows * LD64];
-    __nv_bfloat16 dY[kRows * LD16], dZ2[kRows * LD64], dZ1[kRows * LD64];
-    float Z1[kRows * kHid], Z2[kRows * kHid];
-    float Y[kRows * kOut];
+__device__ __forceinline__ uint32_t pack_bf16(F2 v) {
+    const float2 u = un(v);
+    const __nv_bfloat162 p = __floats2bfloat162_rn(u.x, u.y);
+    return *reinterpret_cast<const uint32_t*>(&p);
+}
+__device__ __forceinline__ F2 biased(const float* c, const float* bias) {
+    const float2 b = *reinterpret_cast<const float2*>(bias);
+    return add2(f2(c[0], c[1]), f2(b.x, b.y));
+}
+__device__ __forceinline__ void clear(float C[4]) { C[0] = C[1] = C[2] = C[3] = 0.f; }
+
+struct WeightSmem {
+    __nv_bfloat16 W1[kHid * LD16], W2[kHid * LD64], W3[kOut * LD64];
     float b1[kHid], b2[kHid], b3[kOut];
 };
 
-__device__ void load_weights(Smem& S, const __nv_bfloat16* __restrict__ W1, const __nv_bfloat16* __restrict__ W2,
-                             const __nv_bfloat16* __restrict__ W3, const float* __restrict__ b1,
-                             const float* __restrict__ b2, const float* __restrict__ b3) {
-    for (int k = threadIdx.x; k < kHid * kIn; k += blockDim.x) S.W1[(k / kIn) * LD16 + k % kIn] = W1[k];
-    for (int k = threadIdx.x; k < kHid * kHid; k += blockDim.x) S.W2[(k / kHid) * LD64 + k % kHid] = W2[k];
-    for (int k = threadIdx.x; k < 16 * kHid; k += blockDim.x)
-        S.W3[(k / kHid) * LD64 + k % kHid] = k < kOut * kHid ? W3[k] : __float2bfloat16_rn(0.f);
-    for (int k = threadIdx.x; k < kHid; k += blockDim.x) {
-        S.b1[k] = b1[k];
-        S.b2[k] = b2[k];
+// By 32 * kWarps threads, all loads of a matrix in flight.
+__device__ __forceinline__ void load_weights(WeightSmem& S, const __nv_bfloat16* __restrict__ W1,
+                                             const __nv_bfloat16* __restrict__ W2, const __nv_bfloat16* __restrict__ W3,
+                                             const float* __restrict__ b1, const float* __restrict__ b2,
+                                             const float* __restrict__ b3) {
+    constexpr int kStep = 32 * kWarps;
+    __nv_bfloat16 r1[kHid * kIn / kStep], r2[kHid * kHid / kStep], r3[kOut * kHid / kStep];
+#pragma unroll
+    for (int i = 0; i < kHid * kHid / kStep; ++i) r2[i] = W2[i * kStep + threadIdx.x];
+#pragma unroll
+    for (int i = 0; i < kHid * kIn / kStep; ++i) r1[i] = W1[i * kStep + threadIdx.x];
+#pragma unroll
+    for (int i = 0; i < kOut * kHid / kStep; ++i) r3[i] = W3[i * kStep + threadIdx.x];
+    if (threadIdx.x < kHid) {
+        S.b1[threadIdx.x] = b1[threadIdx.x];
+        S.b2[threadIdx.x] = b2[threadIdx.x];
     }
     if (threadIdx.x < kOut) S.b3[threadIdx.x] = b3[threadIdx.x];
-    for (int k = threadIdx.x; k < kRows * LD16; k += blockDim.x) S.dY[k] = __float2bfloat16_rn(0.f);
+    const int row = threadIdx.x / kHid, col = threadIdx.x % kHid;
+#pragma unroll
+    for (int i = 0; i < kHid * kHid / kStep; ++i) S.W2[(i * (kStep / kHid) + row) * LD64 + col] = r2[i];
+#pragma unroll
+    for (int i = 0; i < kOut * kHid / kStep; ++i) S.W3[(i * (kStep / kHid) + row) * LD64 + col] = r3[i];
+#pragma unroll
+    for (int i = 0; i < kHid * kIn / kStep; ++i)
+        S.W1[(i * (kStep / kIn) + threadIdx.x / kIn) * LD16 + threadIdx.x % kIn] = r1[i];
 }
 
-// Forward of one warp's 16 points (rows r0..r0+15 of the slice): fills X, Z1, H1, Z2, H2, Y.
-__device__ void warp_forward(Smem& S, const __nv_bfloat16* __restrict__ x, int64_t n, int64_t p0, int r0) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    {   // X rows: 16 rows x 32 bytes, one 16-byte half row per lane
-        const int row = lane >> 1, half = lane & 1;
-        const int64_t p = p0 + row;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (p < n) v = *reinterpret_cast<const uint4*>(x + p * kIn + half * 8);
-        *reinterpret_cast<uint4*>(S.X + (size_t)(r0 + row) * LD16 + half * 8) = v;
-    }
-    __syncwarp();
-    uint32_t a[4];
-    frag_a(a, S.X, LD16, r0, 0);
-#pragma unroll
-    for (int j = 0; j < kHid / 8; ++j) {
-        uint32_t b[2];
-        frag_b(b, S.W1, LD16, 8 * j, 0);
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        mma(c, a, b);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int row = r0 + g + (e >> 1) * 8, col = 8 * j + 2 * t + (e & 1);
-            const float z = c[e] + S.b1[col];
-            S.Z1[row * kHid + col] = z;
-            S.H1[row * LD64 + col] = __float2bfloat16_rn(gelu(z));
-        }
-    }
-    __syncwarp();
-    uint32_t a4[4][4];
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) frag_a(a4[kk], S.H1, LD64, r0, 16 * kk);
-#pragma unroll
-    for (int j = 0; j < kHid / 8; ++j) {
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            uint32_t b[2];
-            frag_b(b, S.W2, LD64, 8 * j, 16 * kk);
-            mma(c, a4[kk], b);
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int row = r0 + g + (e >> 1) * 8, col = 8 * j + 2 * t + (e & 1);
-            const float z = c[e] + S.b2[col];
-            S.Z2[row * kHid + col] = z;
-            S.H2[row * LD64 + col] = __float2bfloat16_rn(gelu(z));
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) frag_a(a4[kk], S.H2, LD64, r0, 16 * kk);
-    float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-        uint32_t b[2];
-        frag_b(b, S.W3, LD64, 0, 16 * kk);
-        mma(c, a4[kk], b);
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int row = r0 + g + (e >> 1) * 8, col = 2 * t + (e & 1);
-        S.Y[row * kOut + col] = c[e] + S.b3[col];
-    }
-    __syncwarp();
+// the words of lane (g, t) of the 16 x 16 A fragment of points sl * 16 ..
+__device__ __forceinline__ void load_points(uint32_t a[4], const __nv_bfloat16* __restrict__ x, int64_t n, int64_t p0) {
+    const int lane = threadIdx.x & 31, t = lane & 3;
+    const uint32_t* __restrict__ xw = reinterpret_cast<const uint32_t*>(x);  // 8 words per point
+    const int64_t pa = p0 + (lane >> 2), pb = pa + 8;
+    a[0] = pa < n ? xw[pa * 8 + t] : 0u;
+    a[1] = pb < n ? xw[pb * 8 + t] : 0u;
+    a[2] = pa < n ? xw[pa * 8 + t + 4] : 0u;
+    a[3] = pb < n ? xw[pb * 8 + t + 4] : 0u;
 }
 
 // Inference: activations never leave registers.  The f32 accumulator fragment of a 16 x 8
-// product tile (rows g, g + 8; columns 2t, 2t + 1 of lane (g, t)) is, after bias and GELU and
-// packing column pairs to bf16x2, exactly the A fragment of the next layer's 16 x 16 k-tile (the
+// product tile (rows g, g + 8; columns 2t, 2t + 1 of lane (g, t)) is, after bias, GELU and
+// packing column pairs to bf16x2 exactly the A fragment of the next layer's 16 x 16 k-tile (the
 // k-tile of columns 16 kk.. is made of n-tiles 2 kk and 2 kk + 1), so each warp carries its 16
 // points through the three layers with no shared-memory round trip; only the weights are staged.
-struct WeightSmem {
-    __nv_bfloat16 W1[kHid * LD16], W2[kHid * LD64], W3[16 * LD64];  // W3 rows 8..15 zero
-    float b1[kHid], b2[kHid], b3[kOut];
-};
+// The FP32 and special-function pipes bound it (56 % and 51 % busy, issue 59 %): 710 us for 6.4 M points with
+// scalar arithmetic and a subnormal path around every special function (issue 83 %), 470 us with packed pairs.
+// Four CTAs an SM: at six or more, with the registers that leaves, 520 us and up.
 
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
-
-// bias + GELU of the eight 16 x 8 accumulator tiles C[j] of a 64-wide layer, packed into the
-// four A fragments of the next layer
-__device__ __forceinline__ void activate(const float C[8][4], const float* __restrict__ bias, int t,
-                                         uint32_t A[4][4]) {
+// bias and GELU of two neighbouring 16 x 8 accumulator tiles, packed into one A fragment of the next layer
+__device__ __forceinline__ void activate(const float C[2][4], const float* bias, uint32_t A[4]) {
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-        const int c0 = 16 * kk + 2 * t, c1 = c0 + 8;
-        A[kk][0] = pack_bf16(gelu(C[2 * kk][0] + bias[c0]), gelu(C[2 * kk][1] + bias[c0 + 1]));
-        A[kk][1] = pack_bf16(gelu(C[2 * kk][2] + bias[c0]), gelu(C[2 * kk][3] + bias[c0 + 1]));
-        A[kk][2] = pack_bf16(gelu(C[2 * kk + 1][0] + bias[c1]), gelu(C[2 * kk + 1][1] + bias[c1 + 1]));
-        A[kk][3] = pack_bf16(gelu(C[2 * kk + 1][2] + bias[c1]), gelu(C[2 * kk + 1][3] + bias[c1 + 1]));
-    }
+    for (int e = 0; e < 4; ++e) A[e] = pack_bf16(gelu2(biased(C[e >> 1] + 2 * (e & 1), bias + 8 * (e >> 1))));
 }
 
-constexpr int kInferWarps = 4;
-
-__global__ void __launch_bounds__(32 * kInferWarps)
+__global__ void __launch_bounds__(32 * kWarps, 4)
 k_mlp_forward(const __nv_bfloat16* __restrict__ x, int64_t n, const __nv_bfloat16* __restrict__ W1,
               const __nv_bfloat16* __restrict__ W2, const __nv_bfloat16* __restrict__ W3,
               const float* __restrict__ b1, const float* __restrict__ b2, const float* __restrict__ b3,
               float* __restrict__ out) {
     __shared__ __align__(16) WeightSmem S;
-    for (int k = threadIdx.x; k < kHid * kIn; k += blockDim.x) S.W1[(k / kIn) * LD16 + k % kIn] = W1[k];
-    for (int k = threadIdx.x; k < kHid * kHid; k += blockDim.x) S.W2[(k / kHid) * LD64 + k % kHid] = W2[k];
-    for (int k = threadIdx.x; k < 16 * kHid; k += blockDim.x)
-        S.W3[(k / kHid) * LD64 + k % kHid] = k < kOut * kHid ? W3[k] : __float2bfloat16_rn(0.f);
-    for (int k = threadIdx.x; k < kHid; k += blockDim.x) {
-        S.b1[k] = b1[k];
-        S.b2[k] = b2[k];
-    }
-    if (threadIdx.x < kOut) S.b3[threadIdx.x] = b3[threadIdx.x];
+    load_weights(S, W1, W2, W3, b1, b2, b3);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const uint32_t* __restrict__ xw = reinterpret_cast<const uint32_t*>(x);  // 8 words per point
-    const int64_t slices = (n + 15) / 16;
-    for (int64_t sl = (int64_t)blockIdx.x * kInferWarps + warp; sl < slices;
-         sl += (int64_t)gridDim.x * kInferWarps) {
-        const int64_t p0 = sl * 16, pa = p0 + g, pb = p0 + g + 8;
-        uint32_t a[4];
-        a[0] = pa < n ? xw[pa * 8 + t] : 0u;
-        a[1] = pb < n ? xw[pb * 8 + t] : 0u;
-        a[2] = pa < n ? xw[pa * 8 + t + 4] : 0u;
-        a[3] = pb < n ? xw[pb * 8 + t + 4] : 0u;
-        float C[8][4];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            uint32_t b[2];
-            frag_b(b, S.W1, LD16, 8 * j, 0);
-            C[j][0] = C[j][1] = C[j][2] = C[j][3] = 0.f;
-            mma(C[j], a, b);
-        }
-        uint32_t A[4][4];
-        activate(C, S.b1, t, A);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            C[j][0] = C[j][1] = C[j][2] = C[j][3] = 0.f;
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                uint32_t b[2];
-                frag_b(b, S.W2, LD64, 8 * j, 16 * kk);
-                mma(C[j], A[kk], b);
-            }
-        }
-        activate(C, S.b2, t, A);
-        float y[4] = {0.f, 0.f, 0.f, 0.f};
+    // four 8 x 8 weight tiles at a time: two products' B fragments, of output tiles j and j + 1 (first layer)
+    // or of k-tiles kk and kk + 1
+    const __nv_bfloat16* const w1 = S.W1 + (size_t)((lane & 7) + (lane >> 4) * 8) * LD16 + ((lane >> 3) & 1) * 8;
+    const __nv_bfloat16* const w2 = S.W2 + (size_t)(lane & 7) * LD64 + (lane >> 3) * 8;
+    const __nv_bfloat16* const w3 = S.W3 + (size_t)(lane & 7) * LD64 + (lane >> 3) * 8;
+    const int64_t slices = (n + 15) / 16, step = (int64_t)gridDim.x * kWarps;
+    int64_t sl = (int64_t)blockIdx.x * kWarps + warp;
+    uint32_t a[4];
+    load_points(a, x, n, sl * 16);
+    for (; sl < slices; sl += step) {
+        uint32_t A[4][4], b[4];
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-            uint32_t b[2];
-            frag_b(b, S.W3, LD64, 0, 16 * kk);
-            mma(y, A[kk], b);
+            float C[2][4];
+            clear(C[0]);
+            clear(C[1]);
+            ldsm_x4(b, w1 + 16 * kk * LD16);
+            mma(C[0], a, b);
+            mma(C[1], a, b + 2);
+            activate(C, S.b1 + 16 * kk + 2 * t, A[kk]);
         }
+        load_points(a, x, n, (sl + step) * 16);  // the next points, while these are carried through
+        float y[4];
+        clear(y);
+        uint32_t b3[4];
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            float C[2][4];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                clear(C[j]);
+#pragma unroll
+                for (int k = 0; k < 4; k += 2) {
+                    ldsm_x4(b, w2 + 8 * (2 * kk + j) * LD64 + 16 * k);
+                    mma(C[j], A[k], b);
+                    mma(C[j], A[k + 1], b + 2);
+                }
+            }
+            uint32_t H[4];
+            activate(C, S.b2 + 16 * kk + 2 * t, H);
+            if (kk % 2 == 0) ldsm_x4(b3, w3 + 16 * kk);
+            mma(y, H, b3 + 2 * (kk % 2));
+        }
+        const int64_t pa = sl * 16 + g, pb = pa + 8;
         const int c = 2 * t;
         if (pa < n) *reinterpret_cast<float2*>(out + pa * kOut + c) = make_float2(y[0] + S.b3[c], y[1] + S.b3[c + 1]);
         if (pb < n) *reinterpret_cast<float2*>(out + pb * kOut + c) = make_float2(y[2] + S.b3[c], y[3] + S.b3[c + 1]);
     }
 }
 
-__global__ void __launch_bounds__(32 * kWarps)
+// What a slice's weight gradients contract over its 64 points, which the four warps exchange: BF16 rows of
+// 4-byte words whose padding puts the fragments' stores and loads on different banks.
+struct SliceSmem {
+    __nv_bfloat16 H1[kRows * LD64], H2[kRows * LD64], dZ2[kRows * LD64], dZ1[kRows * LD64];
+    __nv_bfloat16 X[kRows * LD16], dY[kRows * kOut];
+};
+struct TrainSmem {
+    WeightSmem w;
+    SliceSmem s[2];
+};
+
+__device__ __forceinline__ float quad_sum(float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
+
+// A slice's forward and backward chain stays in a warp's registers (accumulator fragments become the next
+// product's A fragments, the GELU derivatives of the forward pass wait in FP32 registers); shared memory
+// holds only what the weight gradients contract, in two buffers, so that a slice needs one barrier.  With
+// every activation in shared memory, FP32 Z1 and Z2 among them, and the derivative's erf and exponential
+// evaluated again, a pass over 65,536 points took 70 us; 35 us now, two CTAs an SM by registers, bound by latency
+// (issue 22 %): 1,024 slices are 3.4 per CTA.
+__global__ void __launch_bounds__(32 * kWarps, 2)
 k_mlp_train(const __nv_bfloat16* __restrict__ x, const float* __restrict__ target, int64_t n,
             const __nv_bfloat16* __restrict__ W1, const __nv_bfloat16* __restrict__ W2,
             const __nv_bfloat16* __restrict__ W3, const float* __restrict__ b1, const float* __restrict__ b2,
             const float* __restrict__ b3, float* __restrict__ grad, double* __restrict__ loss_sum) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    Smem& S = *reinterpret_cast<Smem*>(s_raw);
-    load_weights(S, W1, W2, W3, b1, b2, b3);
+    TrainSmem& T = *reinterpret_cast<TrainSmem*>(s_raw);
+    WeightSmem& W = T.w;
+    load_weights(W, W1, W2, W3, b1, b2, b3);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int r0 = 16 * warp;
+    const int r0 = 16 * warp, row = r0 + g;
     const float inv_n = 1.0f / (float)n;
-    float accW2[8][4], accW1[2][4], accW3[2][4];
-    float db1[16], db2[16], db3[kOut];
+    // rows of four 8 x 8 tiles for ldmatrix: lanes 8 i .. 8 i + 7 give tile i's
+    const int tr = lane & 7, ti = lane >> 3;
+    const __nv_bfloat16* const w1 = W.W1 + (tr + (ti >> 1) * 8) * LD16 + (ti & 1) * 8;  // n-tiles j, j + 1
+    const __nv_bfloat16* const w2 = W.W2 + tr * LD64 + ti * 8;                          // k-tiles k, k + 1
+    const __nv_bfloat16* const w3 = W.W3 + tr * LD64 + ti * 8;
+    const int back = (tr + (ti & 1) * 8) * LD64 + (ti >> 1) * 8;  // of a transposed pair of n-tiles, 16 rows
+    float accW2[8][4], accW1[2][4], accW3[4];
+    F2 db1[8], db2[8];  // columns 8 j + 2 t, + 1
+    float db3[2] = {0.f, 0.f};
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) accW2[j][e] = 0.f;
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) accW1[j][e] = accW3[j][e] = 0.f;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) db1[k] = db2[k] = 0.f;
-#pragma unroll
-    for (int k = 0; k < kOut; ++k) db3[k] = 0.f;
+    for (int j = 0; j < 8; ++j) {
+        clear(accW2[j]);
+        db1[j] = db2[j] = f2(0.f);
+    }
+    clear(accW1[0]);
+    clear(accW1[1]);
+    clear(accW3);
     double lsum = 0.0;
 
-    for (int64_t p0 = (int64_t)blockIdx.x * kRows; p0 < n; p0 += (int64_t)gridDim.x * kRows) {
-        warp_forward(S, x, n, p0 + r0, r0);
-        // loss head: lane = point of the warp
-        if (lane < 16) {
-            const int row = r0 + lane;
-            const int64_t p = p0 + row;
-            float dy[kOut] = {0, 0, 0, 0, 0, 0, 0, 0};
-            if (p < n) {
-                const float* y = S.Y + row * kOut;
-                const float* tg = target + p * kOut;
-                float L = 0.f;
-                for (int k = 0; k < 3; ++k) {
-                    const float d = y[k] - tg[k];
-                    L += d * d;
-                    dy[k] = 2.f * d * inv_n;
-                }
-                const float qn = sqrtf(y[3] * y[3] + y[4] * y[4] + y[5] * y[5] + y[6] * y[6]);
-                const float iq = qn > 0.f ? 1.0f / qn : 0.f;
-                float f = 0.f;
-                for (int k = 0; k < 4; ++k) f += y[3 + k] * iq * tg[3 + k];
-                L += 1.f - f * f;
-                float dq[4], dot = 0.f;
-                for (int k = 0; k < 4; ++k) {
-                    dq[k] = -2.f * f * tg[3 + k];
-                    dot += dq[k] * y[3 + k] * iq;
-                }
-                for (int k = 0; k < 4; ++k) dy[3 + k] = (dq[k] - y[3 + k] * iq * dot) * iq * inv_n;
-                const float d = y[7] - tg[7];
-                L += d * d;
-                dy[7] = 2.f * d * inv_n;
-                lsum += (double)L;
-            }
-            for (int k = 0; k < kOut; ++k) {
-                db3[k] += dy[k];
-                S.dY[row * LD16 + k] = __float2bfloat16_rn(dy[k]);
-            }
+    int buf = 0;
+    uint32_t a[4];
+    float tg[2][2];
+    auto fetch = [&](int64_t p) {
+        load_points(a, x, n, p + r0);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                tg[r][c] = p + row + 8 * r < n ? target[(p + row + 8 * r) * kOut + 2 * t + c] : 0.f;
+    };
+    const int64_t step = (int64_t)gridDim.x * kRows;
+    fetch((int64_t)blockIdx.x * kRows);
+    for (int64_t p0 = (int64_t)blockIdx.x * kRows; p0 < n; p0 += step, buf ^= 1) {
+        SliceSmem& S = T.s[buf];
+        uint32_t b[4], A[4][4];
+        const bool in[2] = {p0 + row < n, p0 + row + 8 < n};
+        // word e of an A fragment at columns c0..: rows row, row + 8, then the same 8 columns on
+        auto put = [&](__nv_bfloat16* M, int ld, int c0, const uint32_t w[4]) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                *reinterpret_cast<uint32_t*>(M + (row + 8 * (e & 1)) * ld + c0 + 8 * (e >> 1) + 2 * t) = w[e];
+        };
+        put(S.X, LD16, 0, a);
+        F2 g1[4][4], g2[4][4];  // gelu' at the pairs of the fragments' words
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            float C[2][4];
+            clear(C[0]);
+            clear(C[1]);
+            ldsm_x4(b, w1 + 16 * kk * LD16);
+            mma(C[0], a, b);
+            mma(C[1], a, b + 2);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                A[kk][e] = pack_bf16(
+                    gelu2(biased(C[e >> 1] + 2 * (e & 1), W.b1 + 16 * kk + 8 * (e >> 1) + 2 * t), g1[kk][e]));
+            put(S.H1, LD64, 16 * kk, A[kk]);
         }
-        __syncwarp();
+        float y[4];
+        clear(y);
+        uint32_t bw[4];
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            float C[2][4];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                clear(C[j]);
+#pragma unroll
+                for (int k = 0; k < 4; k += 2) {
+                    ldsm_x4(b, w2 + 8 * (2 * kk + j) * LD64 + 16 * k);
+                    mma(C[j], A[k], b);
+                    mma(C[j], A[k + 1], b + 2);
+                }
+            }
+            uint32_t H[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                H[e] = pack_bf16(
+                    gelu2(biased(C[e >> 1] + 2 * (e & 1), W.b2 + 16 * kk + 8 * (e >> 1) + 2 * t), g2[kk][e]));
+            put(S.H2, LD64, 16 * kk, H);
+            if (kk % 2 == 0) ldsm_x4(bw, w3 + 16 * kk);
+            mma(y, H, bw + 2 * (kk % 2));
+        }
+        // loss head: the four lanes of a row hold its outputs 2 t, 2 t + 1; 3..6 are the quaternion
+        const bool qa = t >= 2, qb = t == 1 || t == 2;
+        uint32_t dyw[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const float ya = y[2 * r] + W.b3[2 * t], yb = y[2 * r + 1] + W.b3[2 * t + 1];
+            const float qn = sqrtf(quad_sum((qa ? ya * ya : 0.f) + (qb ? yb * yb : 0.f)));
+            const float iq = qn > 0.f ? 1.0f / qn : 0.f;
+            const float ua = ya * iq, ub = yb * iq;
+            const float f = quad_sum((qa ? ua * tg[r][0] : 0.f) + (qb ? ub * tg[r][1] : 0.f));
+            const float dqa = -2.f * f * tg[r][0], dqb = -2.f * f * tg[r][1];
+            const float dot = quad_sum((qa ? dqa * ua : 0.f) + (qb ? dqb * ub : 0.f));
+            const float da = ya - tg[r][0], db = yb - tg[r][1];
+            float dya = qa ? (dqa - ua * dot) * iq * inv_n : 2.f * da * inv_n;
+            float dyb = qb ? (dqb - ub * dot) * iq * inv_n : 2.f * db * inv_n;
+            if (!in[r]) dya = dyb = 0.f;
+            if (in[r]) lsum += (double)((qa ? 0.f : da * da) + (qb ? 0.f : db * db) + (t == 0 ? 1.f - f * f : 0.f));
+            db3[0] += dya;
+            db3[1] += dyb;
+            dyw[r] = pack_bf16(f2(dya, dyb));
+            *reinterpret_cast<uint32_t*>(S.dY + (row + 8 * r) * kOut + 2 * t) = dyw[r];
+        }
+        fetch(p0 + step);  // the next slice's, under the backward pass
         // dZ2 = (dY W3) gelu'(Z2)
-        uint32_t a[4];
-        frag_a(a, S.dY, LD16, r0, 0);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            uint32_t b[2];
-            frag_b_t(b, S.W3, LD64, 0, 8 * j);
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
-            mma(c, a, b);
+        for (int kk = 0; kk < 4; ++kk) {
+            if (kk % 2 == 0) ldsm_x4_t(bw, w3 + 16 * kk);
+            float C[2][4];
+            clear(C[0]);
+            clear(C[1]);
+            mma_k8(C[0], dyw, bw[2 * (kk % 2)]);
+            mma_k8(C[1], dyw, bw[2 * (kk % 2) + 1]);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int row = r0 + g + (e >> 1) * 8, col = 8 * j + 2 * t + (e & 1);
-                const float dz = c[e] * gelu_d(S.Z2[row * kHid + col]);
-                db2[2 * j + (e & 1)] += dz;
-                S.dZ2[row * LD64 + col] = __float2bfloat16_rn(dz);
+                const float* c = C[e >> 1] + 2 * (e & 1);
+                const F2 dz = mul2(f2(c[0], c[1]), g2[kk][e]);
+                db2[2 * kk + (e >> 1)] = add2(db2[2 * kk + (e >> 1)], dz);
+                A[kk][e] = pack_bf16(dz);
             }
+            put(S.dZ2, LD64, 16 * kk, A[kk]);
         }
-        __syncwarp();
         // dZ1 = (dZ2 W2) gelu'(Z1)
-        uint32_t a4[4][4];
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) frag_a(a4[kk], S.dZ2, LD64, r0, 16 * kk);
+        for (int kk = 0; kk < 4; ++kk) {
+            float C[2][4];
+            clear(C[0]);
+            clear(C[1]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                uint32_t b[2];
-                frag_b_t(b, S.W2, LD64, 16 * kk, 8 * j);
-                mma(c, a4[kk], b);
+            for (int k = 0; k < 4; ++k) {
+                ldsm_x4_t(b, W.W2 + back + 16 * k * LD64 + 16 * kk);
+                mma(C[0], A[k], b);
+                mma(C[1], A[k], b + 2);
             }
+            uint32_t D[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int row = r0 + g + (e >> 1) * 8, col = 8 * j + 2 * t + (e & 1);
-                const float dz = c[e] * gelu_d(S.Z1[row * kHid + col]);
-                db1[2 * j + (e & 1)] += dz;
-                S.dZ1[row * LD64 + col] = __float2bfloat16_rn(dz);
+                const float* c = C[e >> 1] + 2 * (e & 1);
+                const F2 dz = mul2(f2(c[0], c[1]), g1[kk][e]);
+                db1[2 * kk + (e >> 1)] = add2(db1[2 * kk + (e >> 1)], dz);
+                D[e] = pack_bf16(dz);
             }
+            put(S.dZ1, LD64, 16 * kk, D);
         }
+        // The other buffer's readers are done: each warp came here after its products of the slice before.
         __syncthreads();
-        // weight gradients over the slice's 64 points (K = data rows)
+        // weight gradients over the slice's 64 points: this warp's 16 rows of dW2 and dW1, and columns of dW3
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
             uint32_t at[4];
-            frag_a_t(at, S.dZ2, LD64, 16 * kk, 16 * warp);  // rows of dW2 owned by this warp
+            frag_a_t(at, S.dZ2, LD64, 16 * kk, r0);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                uint32_t b[2];
-                frag_b_t(b, S.H1, LD64, 16 * kk, 8 * j);
+            for (int j = 0; j < 8; j += 2) {
+                ldsm_x4_t(b, S.H1 + back + 16 * kk * LD64 + 8 * j);
                 mma(accW2[j], at, b);
+                mma(accW2[j + 1], at, b + 2);
             }
-            frag_a_t(at, S.dZ1, LD64, 16 * kk, 16 * warp);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                uint32_t b[2];
-                frag_b_t(b, S.X, LD16, 16 * kk, 8 * j);
-                mma(accW1[j], at, b);
-            }
-            frag_a_t(at, S.dY, LD16, 16 * kk, 0);  // dY^T padded to 16 rows
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                uint32_t b[2];
-                frag_b_t(b, S.H2, LD64, 16 * kk, 8 * (2 * warp + j));
-                mma(accW3[j], at, b);
-            }
+            frag_a_t(at, S.dZ1, LD64, 16 * kk, r0);
+            ldsm_x4_t(b, S.X + (16 * kk + tr + (ti & 1) * 8) * LD16 + (ti >> 1) * 8);
+            mma(accW1[0], at, b);
+            mma(accW1[1], at, b + 2);
+            frag_a_t(at, S.H2, LD64, 16 * kk, r0);  // transposed: rows are hidden units, columns outputs
+            ldsm_x2_t(b, S.dY + (16 * kk + tr + (ti & 1) * 8) * kOut);
+            mma(accW3, at, b);
         }
-        __syncthreads();
     }
     // flush: weight gradients (C fragment rows g / g + 8, cols 2t, 2t + 1)
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
+    for (int e = 0; e < 4; ++e) {
+        const int m = row + (e >> 1) * 8, c = 2 * t + (e & 1);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int m = 16 * warp + g + (e >> 1) * 8, col = 8 * j + 2 * t + (e & 1);
-            atomicAdd(&grad[oW2 + m * kHid + col], accW2[j][e]);
-        }
+        for (int j = 0; j < 8; ++j) atomicAdd(&grad[oW2 + m * kHid + 8 * j + c], accW2[j][e]);
 #pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int m = 16 * warp + g + (e >> 1) * 8, col = 8 * j + 2 * t + (e & 1);
-            atomicAdd(&grad[oW1 + m * kIn + col], accW1[j][e]);
-            if (e < 2) {  // dW3 has 8 rows: the fragment's upper half
-                const int col3 = 8 * (2 * warp + j) + 2 * t + (e & 1);
-                atomicAdd(&grad[oW3 + g * kHid + col3], accW3[j][e]);
-            }
-        }
-    // bias gradients: reduce over the lanes sharing t (rows), then over lanes (db3)
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        for (int o = 4; o < 32; o <<= 1) {
-            db1[k] += __shfl_xor_sync(0xffffffffu, db1[k], o);
-            db2[k] += __shfl_xor_sync(0xffffffffu, db2[k], o);
-        }
+        for (int j = 0; j < 2; ++j) atomicAdd(&grad[oW1 + m * kIn + 8 * j + c], accW1[j][e]);
+        atomicAdd(&grad[oW3 + c * kHid + m], accW3[e]);
     }
-    if (g == 0) {
+    // bias gradients: reduce over the lanes sharing t (rows)
+    auto rows_sum = [&](float v) {
+        for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
+    for (int j = 0; j < 8; ++j) {
+        const float2 u = un(db1[j]), v = un(db2[j]);
+        const float s[4] = {rows_sum(u.x), rows_sum(u.y), rows_sum(v.x), rows_sum(v.y)};
+        if (g == 0)
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                atomicAdd(&grad[ob1 + 8 * j + 2 * t + q], db1[2 * j + q]);
-                atomicAdd(&grad[ob2 + 8 * j + 2 * t + q], db2[2 * j + q]);
+                atomicAdd(&grad[ob1 + 8 * j + 2 * t + q], s[q]);
+                atomicAdd(&grad[ob2 + 8 * j + 2 * t + q], s[2 + q]);
             }
     }
 #pragma unroll
-    for (int k = 0; k < kOut; ++k)
-        for (int o = 1; o < 32; o <<= 1) db3[k] += __shfl_xor_sync(0xffffffffu, db3[k], o);
-    if (lane == 0)
-        for (int k = 0; k < kOut; ++k) atomicAdd(&grad[ob3 + k], db3[k]);
+    for (int q = 0; q < 2; ++q) {
+        const float s = rows_sum(db3[q]);
+        if (g == 0) atomicAdd(&grad[ob3 + 2 * t + q], s);
+    }
     for (int o = 1; o < 32; o <<= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
     if (lane == 0) atomicAdd(loss_sum, lsum);
 }
@@ -502,7 +519,7 @@ int grid_for(int64_t n) {
 
 void enable_smem() {
     static bool done = [] {
-        cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+        cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem));
         return true;
     }();
     (void)done;
@@ -520,12 +537,12 @@ int launch_mlp_forward(const void* x, int64_t n, const float* master, const void
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_forward, 32 * kInferWarps, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_forward, 32 * kWarps, 0);
         return sms * (per_sm > 0 ? per_sm : 1);
     }();
     const int64_t slices = (n + 15) / 16;
-    const int64_t blocks = std::min<int64_t>(grid, (slices + kInferWarps - 1) / kInferWarps);
-    k_mlp_forward<<<(unsigned)blocks, 32 * kInferWarps, 0, s>>>(
+    const int64_t blocks = std::min<int64_t>(grid, (slices + kWarps - 1) / kWarps);
+    k_mlp_forward<<<(unsigned)blocks, 32 * kWarps, 0, s>>>(
         static_cast<const __nv_bfloat16*>(x), n, static_cast<const __nv_bfloat16*>(W1),
         static_cast<const __nv_bfloat16*>(W2), static_cast<const __nv_bfloat16*>(W3), master + ob1,
         master + ob2, master + ob3, out);
@@ -536,7 +553,7 @@ int launch_mlp_train(const void* x, const float* target, int64_t n, const float*
                      const void* W2, const void* W3, float* grad, double* loss_sum, cudaStream_t s) {
     if (n <= 0) return 0;
     enable_smem();
-    k_mlp_train<<<grid_for(n), 32 * kWarps, sizeof(Smem), s>>>(
+    k_mlp_train<<<grid_for(n), 32 * kWarps, sizeof(TrainSmem), s>>>(
         static_cast<const __nv_bfloat16*>(x), target, n, static_cast<const __nv_bfloat16*>(W1),
         static_cast<const __nv_bfloat16*>(W2), static_cast<const __nv_bfloat16*>(W3), master + ob1,
         master + ob2, master + ob3, grad, loss_sum);
