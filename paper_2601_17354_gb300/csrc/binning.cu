@@ -206,79 +206,45 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
     return x;
 }
 
-// Reach mask of one entry per lane (warp-collective): tiles of the super-tile at tile (bx, by) (each
-// lane its own) that Gaussian g reaches, bit (ty - by) kSuperW + tx - bx.  Rectangles of <= 32 tiles: read row by row
-// from the projection's reach mask.  Larger ones: the warp runs the projection's reach test over
-// all such lanes' candidate tiles together, 32 per round (candidate k by lane k mod 32, its lane
-// found by a shuffle binary search over the lanes' inclusive candidate counts), so one large
-// Gaussian does not hold its warp for 32 tests.
-__device__ __forceinline__ uint32_t entry_mask(bool valid, uint32_t g, uint2 r, uint32_t hm, uint32_t bx, uint32_t by,
-                                               int T, const Scratch& sc, int lane, uint32_t* s_big) {
-    uint32_t mask = 0, ncand = 0, X0 = 0, Y0 = 0, wX = 1;
-    float u = 0.f, v = 0.f, ca = 0.f, cb = 0.f, cc = 0.f, ssx = 0.f, ssy = 0.f;
-    if (valid) {
-        const uint32_t x0 = r.x & 0xffffu, y0 = r.x >> 16, x1 = r.y & 0xffffu, y1 = r.y >> 16;
-        X0 = max(x0, bx);
-        Y0 = max(y0, by);
-        const uint32_t X1 = min(x1, bx + kSuperW), Y1 = min(y1, by + kSuperH);
-        const uint32_t w = x1 - x0;
-        wX = X1 - X0;  // >= 1: the super-tile lies in the Gaussian's super-tile rectangle
-        if (w * (y1 - y0) <= 32u) {
-            const uint32_t row = (1u << wX) - 1u;
-            for (uint32_t ty = Y0; ty < Y1; ++ty)
-                mask |= ((hm >> ((ty - y0) * w + (X0 - x0))) & row) << ((ty - by) * kSuperW + (X0 - bx));
-        } else {
-            ncand = wX * (Y1 - Y0);
-            const float4 p = sc.xyo[g], q = sc.conic[g];
-            u = p.x;
-            v = p.y;
-            ca = q.x;
-            cb = q.y;
-            cc = q.z;
-            ssx = __fdiv_rn(q.y, q.x);
-            ssy = __fdiv_rn(q.y, q.z);
+// Reach masks of entries without one of the projection's (rectangles of more than 32 tiles over more than 2 x 2
+// super-tiles), warp-collective: tiles of the super-tile at tile (bx, by) (each lane its own) that Gaussian g
+// reaches, bit (ty - by) kSuperW + tx - bx; 0 for lanes without `need`.  The warp runs the projection's
+// reach test over all such lanes' candidate tiles together, 32 per round (candidate k by lane k mod 32), so one
+// large Gaussian does not hold its warp for 32 tests.
+struct BigSmem {
+    uint32_t mask[32], lane[32];
+    uint4 cand[32];  // first candidate, tile x0 | y0 << 16 of the part inside the super-tile, its width, Gaussian
+};
+__device__ __forceinline__ uint32_t entry_mask(bool need, uint32_t g, uint2 r, uint32_t bx, uint32_t by, int T,
+                                               const Scratch& sc, int lane, BigSmem& S) {
+    if (!__any_sync(kFull, need)) return 0u;
+    uint32_t X0 = 0, Y0 = 0, w = 0, ncand = 0;
+    if (need) {
+        X0 = max(r.x & 0xffffu, bx);
+        Y0 = max(r.x >> 16, by);
+        w = min(r.y & 0xffffu, bx + kSuperW) - X0;  // >= 1: the super-tile lies in the Gaussian's super-tile rectangle
+        ncand = w * (min(r.y >> 16, by + kSuperH) - Y0);
+    }
+    WarpRuns runs(ncand);
+    S.mask[lane] = 0u;
+    if (need) {
+        S.lane[runs.rank] = (uint32_t)lane;
+        S.cand[runs.rank] = make_uint4(runs.first, X0 | (Y0 << 16), w, g);
+    }
+    __syncwarp();
+    for (uint32_t b = 0; b < runs.total; b += 32) {
+        const uint32_t o = runs.owner(b), k = b + (uint32_t)lane;
+        if (k < runs.total) {
+            const uint4 c = S.cand[o];
+            const uint32_t local = k - c.x, dy = local / c.z, dx = local - dy * c.z;
+            const uint32_t tx = (c.y & 0xffffu) + dx, ty = (c.y >> 16) + dy;
+            const float4 p = sc.xyo[c.w], q = sc.conic[c.w];
+            if (tile_hit(p.x, p.y, q.x, q.y, q.z, __fdiv_rn(q.y, q.x), __fdiv_rn(q.y, q.z), (int)tx, (int)ty, (float)T))
+                atomicOr(&S.mask[S.lane[o]], 1u << ((ty % kSuperH) * kSuperW + tx % kSuperW));
         }
     }
-    uint32_t incl = ncand;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-    }
-    const uint32_t total = __shfl_sync(kFull, incl, 31), first = incl - ncand;
-    if (total) {  // warp-uniform
-        s_big[lane] = 0u;
-        __syncwarp();
-        for (uint32_t b = 0; b < total; b += 32) {
-            const uint32_t k = b + (uint32_t)lane;
-            int lo = 0, hi = 31;  // owner of candidate k: the first lane whose inclusive count exceeds k
-#pragma unroll
-            for (int step = 0; step < 5; ++step) {
-                const int mid = (lo + hi) >> 1;
-                const uint32_t im = __shfl_sync(kFull, incl, mid);
-                if (lo < hi) {
-                    if (im > k) hi = mid;
-                    else lo = mid + 1;
-                }
-            }
-            const uint32_t of = __shfl_sync(kFull, first, lo), ow = __shfl_sync(kFull, wX, lo);
-            const uint32_t ox = __shfl_sync(kFull, X0, lo), oy = __shfl_sync(kFull, Y0, lo);
-            const float ou = __shfl_sync(kFull, u, lo), ov = __shfl_sync(kFull, v, lo);
-            const float oa = __shfl_sync(kFull, ca, lo), ob = __shfl_sync(kFull, cb, lo), oc = __shfl_sync(kFull, cc, lo);
-            const float osx = __shfl_sync(kFull, ssx, lo), osy = __shfl_sync(kFull, ssy, lo);
-            const uint32_t obx = __shfl_sync(kFull, bx, lo), oby = __shfl_sync(kFull, by, lo);  // owner's super-tile
-            if (k < total) {
-                const uint32_t local = k - of, dy = local / ow, dx = local - dy * ow;
-                const uint32_t tx = ox + dx, ty = oy + dy;
-                if (tile_hit(ou, ov, oa, ob, oc, osx, osy, (int)tx, (int)ty, T))
-                    atomicOr(&s_big[lo], 1u << ((ty - oby) * kSuperW + (tx - obx)));
-            }
-        }
-        __syncwarp();
-        mask |= s_big[lane];
-        __syncwarp();
-    }
-    return mask;
+    __syncwarp();
+    return S.mask[lane];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -287,111 +253,86 @@ __device__ __forceinline__ uint32_t entry_mask(bool valid, uint32_t g, uint2 r, 
 // e0 the Gaussian's canonical index and its reach mask of the super-tile (rectangles of <= 32
 // tiles: read from their reach bits; larger ones whose super-tile rectangle spans at most 2 x 2:
 // the projection's masks; the rest: entry_mask).  Each warp walks
-// the entries of its own 32 Gaussians, 32 per round (entry k by lane k mod 32; its Gaussian found
-// by a shuffle binary search over the lanes' inclusive entry counts).
+// the entries of its own 32 Gaussians, 32 per round (entry k by lane k mod 32), whose records it
+// keeps in shared memory by rank.
 // ---------------------------------------------------------------------------------------------
+struct CoarseRec {
+    uint4 a;  // rectangle, hitmask, Gaussian
+    uint4 b;  // first entry, super-tiles across | how << 30, super-tiles of a row of the grid, first super-tile
+    uint4 m;  // the projection's masks (how = 0)
+};
 __global__ void __launch_bounds__(kProjBlock)
 k_coarse_emit(int64_t n, int SX, int T, int64_t capacity, const uint32_t* __restrict__ perm, Scratch sc,
               uint32_t* __restrict__ gidx, uint32_t* __restrict__ gmask, int passes, uint32_t last_mask,
               const RenderDesc* __restrict__ renders, int R) {
     pdl_begin();
-    __shared__ uint32_t s_sx0[kProjBlock], s_sy0[kProjBlock], s_sw[kProjBlock];
-    __shared__ uint32_t s_SX[kProjBlock], s_base[kProjBlock], s_gid[kProjBlock], s_hm[kProjBlock];
-    __shared__ uint2 s_rect[kProjBlock];
-    __shared__ uint4 s_sm[kProjBlock];
+    __shared__ CoarseRec s_rec[kProjBlock];
     __shared__ uint32_t s_warp[kProjBlock / 32];
-    __shared__ uint32_t s_big[kProjBlock / 32][32];
+    __shared__ BigSmem s_big[kProjBlock / 32];
     __shared__ uint32_t s_hist[4][kRadix];  // digit counts of the written keys, pass by pass
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t i = (int64_t)blockIdx.x * kProjBlock + t;
-    for (int k = t; k < 4 * kRadix; k += kProjBlock) (&s_hist[0][0])[k] = 0u;
-    uint32_t cnt = 0;
-    if (i < n) {
-        const uint32_t g = perm[i];
-        s_gid[t] = g;
-        if (sc.touched[g]) {
-            const uint2 r = sc.rect[g];
-            uint32_t sx0, sy0, sx1, sy1;
-            super_rect(r, sx0, sy0, sx1, sy1);
-            s_sx0[t] = sx0;
-            s_sy0[t] = sy0;
-            s_sw[t] = sx1 - sx0;
-            cnt = (sx1 - sx0) * (sy1 - sy0);
-            s_rect[t] = r;
-            const uint32_t area = ((r.y & 0xffffu) - (r.x & 0xffffu)) * ((r.y >> 16) - (r.x >> 16));
-            s_hm[t] = area <= 32u ? sc.hitmask[g] : 0u;
-            if (area <= 32u) s_sw[t] |= 0x40000000u;                          // masks from hitmask
-            else if (sx1 - sx0 <= 2u && sy1 - sy0 <= 2u) s_sm[t] = sc.smask[g];  // projection's masks
-            else s_sw[t] |= 0x80000000u;                                      // entry_mask
-            s_SX[t] = (uint32_t)SX;
-            s_base[t] = 0;
-            if (renders) {  // batch: item g belongs to the last render whose first item is <= g
-                int lo = 0, hi = R - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (renders[mid].item_base <= (int64_t)g) lo = mid;
-                    else hi = mid - 1;
-                }
-                s_SX[t] = (uint32_t)renders[lo].SX;
-                s_base[t] = (uint32_t)renders[lo].super_base;
+    for (int k = t; k < passes * kRadix; k += kProjBlock) (&s_hist[0][0])[k] = 0u;
+    const uint32_t g = i < n ? perm[i] : 0u;
+    const uint32_t reached = i < n ? sc.touched[g] : 0u;
+    uint2 r = make_uint2(0u, 0u);
+    uint32_t cnt = 0, w = 1, how = 0, hm = 0;
+    if (reached) {
+        r = sc.rect[g];
+        uint32_t sx0, sy0, sx1, sy1;
+        super_rect(r, sx0, sy0, sx1, sy1);
+        w = sx1 - sx0;
+        cnt = w * (sy1 - sy0);
+        const uint32_t area = ((r.y & 0xffffu) - (r.x & 0xffffu)) * ((r.y >> 16) - (r.x >> 16));
+        how = area <= 32u ? 1u : w <= 2u && sy1 - sy0 <= 2u ? 0u : 2u;  // hitmask, the projection's masks, entry_mask
+        if (how == 1u) hm = sc.hitmask[g];
+    }
+    WarpRuns runs(cnt);
+    CoarseRec* const recs = s_rec + 32 * warp;
+    if (reached) {
+        CoarseRec& o = recs[runs.rank];
+        o.a = make_uint4(r.x, r.y, hm, g);
+        uint32_t sx = (uint32_t)SX, first_super = 0;
+        if (renders) {  // batch: item g belongs to the last render whose first item is <= g
+            int lo = 0, hi = R - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (renders[mid].item_base <= (int64_t)g) lo = mid;
+                else hi = mid - 1;
             }
+            sx = (uint32_t)renders[lo].SX;
+            first_super = (uint32_t)renders[lo].super_base;
         }
+        o.b = make_uint4(runs.first, w | (how << 30), sx, first_super);
+        if (how == 0u) o.m = sc.smask[g];
     }
-    uint32_t incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += v;
-    }
-    const uint32_t first = incl - cnt;
-    const uint32_t total = __shfl_sync(kFull, incl, 31);
-    if (lane == 31) s_warp[warp] = incl;
+    if (lane == 0) s_warp[warp] = runs.total;
     __syncthreads();  // also publishes the lanes' records in shared memory
     uint32_t before = 0;
 #pragma unroll
-    for (int w = 0; w < kProjBlock / 32; ++w) before += w < warp ? s_warp[w] : 0u;
+    for (int k = 0; k < kProjBlock / 32; ++k) before += k < warp ? s_warp[k] : 0u;
     const unsigned long long out = sc.block_offsets[blockIdx.x] + before;
     uint32_t* ck = reinterpret_cast<uint32_t*>(sc.keys[0]);
-    for (uint32_t b = 0; b < total; b += 32) {  // warp-uniform
+    for (uint32_t b = 0; b < runs.total; b += 32) {  // warp-uniform
         const uint32_t k = b + (uint32_t)lane;
-        int lo = 0, hi = 31;  // owner of entry k: the first lane whose inclusive count exceeds k
-#pragma unroll
-        for (int step = 0; step < 5; ++step) {
-            const int mid = (lo + hi) >> 1;
-            const uint32_t im = __shfl_sync(kFull, incl, mid);
-            if (lo < hi) {
-                if (im > k) hi = mid;
-                else lo = mid + 1;
-            }
-        }
-        const uint32_t ofirst = __shfl_sync(kFull, first, lo);
-        const bool valid = k < total;
-        const int o = warp * 32 + lo;
-        uint32_t sx = 0, sy = 0, slot = 0, g = 0, how = 0;
-        uint2 r = make_uint2(0u, 0u);
-        uint32_t hm = 0;
-        if (valid) {
-            const uint32_t local = k - ofirst, w = s_sw[o] & 0x3fffffffu;
-            const uint32_t dy = local / w, dx = local - dy * w;
-            sx = s_sx0[o] + dx;
-            sy = s_sy0[o] + dy;
-            slot = 2u * dy + dx;
-            g = s_gid[o];
-            how = s_sw[o] >> 30;  // 1: hitmask, 0: projection's masks, 2: entry_mask
-            r = s_rect[o];
-            hm = s_hm[o];
-        }
-        uint32_t mask = entry_mask(valid && how == 2u, g, r, hm, sx * kSuperW, sy * kSuperH, T, sc, lane, s_big[warp]);
-        if (valid && how == 1u)
-            mask = super_mask_from_hits(hm, r.x & 0xffffu, r.x >> 16, r.y & 0xffffu, r.y >> 16, sx, sy);
-        else if (valid && how == 0u)
-            mask = smask_slot(s_sm[o], slot);
+        const CoarseRec& o = recs[runs.owner(b)];
+        const bool valid = k < runs.total;
+        const uint4 ra = o.a, rb = o.b;
+        const uint32_t ow = rb.y & 0x3fffffffu, kind = valid ? rb.y >> 30 : 3u;
+        const uint32_t local = k - rb.x, dy = ow == 1u ? local : local / ow, dx = local - dy * ow;
+        const uint32_t sx = (ra.x & 0xffffu) / kSuperW + dx, sy = (ra.x >> 16) / kSuperH + dy;
+        const uint2 rect = make_uint2(ra.x, ra.y);
+        uint32_t mask = entry_mask(kind == 2u, ra.w, rect, sx * kSuperW, sy * kSuperH, T, sc, lane, s_big[warp]);
+        if (kind == 1u)
+            mask = super_mask_from_hits(ra.z, rect.x & 0xffffu, rect.x >> 16, rect.y & 0xffffu, rect.y >> 16, sx, sy);
+        else if (kind == 0u)
+            mask = smask_slot(o.m, 2u * dy + dx);
         const unsigned long long pos = out + k;
         if (valid && pos < (unsigned long long)capacity) {
-            const uint32_t key = s_base[o] + sy * s_SX[o] + sx;
+            const uint32_t key = rb.w + sy * rb.z + sx;
             ck[pos] = key;
             sc.vals[0][pos] = (uint32_t)pos;
-            gidx[pos] = g;
+            gidx[pos] = ra.w;
             gmask[pos] = mask;
             for (int p = 0; p < passes; ++p)
                 atomicAdd(&s_hist[p][(key >> (p * kRadixBits)) & (p == passes - 1 ? last_mask : kRadix - 1)], 1u);

@@ -28,7 +28,6 @@
 #include <cstdlib>
 #include <type_traits>
 
-#include "f32x2.cuh"
 #include "pgs_internal.cuh"
 
 namespace pgs {

@@ -16,7 +16,6 @@
 // BF16 rounding points: X, weights, H1, H2 and the gradients fed to products (dY, dZ2, dZ1).
 #include <cuda_bf16.h>
 
-#include "f32x2.cuh"
 #include "pgs_internal.cuh"
 
 namespace pgs {

@@ -6,6 +6,7 @@
 
 #include <utility>
 
+#include "f32x2.cuh"
 #include "pocketgs.h"
 
 namespace pgs {
@@ -344,25 +345,69 @@ int launch_loss_dssim(const float* image, const float* target, int W, int H, flo
 // box is at the clamped centre or on an edge at the clamped line minimum.  Part of the prescribed
 // fp32 decision path (membership): every operation an explicit correctly rounded intrinsic, in
 // the order of the oracle's definition.
-__device__ __forceinline__ float hit_q(float X, float Y, float u, float v, float ca, float cb, float cc) {
+__device__ __forceinline__ float hit_q(float X, float Y, float u, float v, float ca, float cb2, float cc) {
     const float dx = __fadd_rn(X, -u), dy = __fadd_rn(Y, -v);
-    return __fadd_rn(__fadd_rn(__fmul_rn(__fmul_rn(ca, dx), dx), __fmul_rn(__fmul_rn(__fadd_rn(cb, cb), dx), dy)),
+    return __fadd_rn(__fadd_rn(__fmul_rn(__fmul_rn(ca, dx), dx), __fmul_rn(__fmul_rn(cb2, dx), dy)),
                      __fmul_rn(__fmul_rn(cc, dy), dy));
 }
-// (sx, sy) = (cb / ca, cb / cc): the slopes of the line minima, per Gaussian; the test stops at the
-// first candidate within the ellipse (min <= 9 exactly when some candidate is)
+__device__ __forceinline__ float2 hit_q2(F2 dx, F2 dy, F2 ca, F2 cb2, F2 cc) {
+    return un(add2(add2(mul2(mul2(ca, dx), dx), mul2(mul2(cb2, dx), dy)), mul2(mul2(cc, dy), dy)));
+}
+// (sx, sy) = (cb / ca, cb / cc): the slopes of the line minima, per Gaussian.  Opposite edges go through one
+// packed instruction each (it rounds as the scalar one); the coordinates are exact below 2^23.  A warp's lanes hardly
+// ever agree on a first candidate inside, so all five are evaluated without branches.
 __device__ __forceinline__ bool tile_hit(float u, float v, float ca, float cb, float cc, float sx, float sy, int tx,
-                                         int ty, int T) {
-    const float xl = __fadd_rn((float)(tx * T), 0.5f), xh = __fadd_rn((float)(tx * T + T), -0.5f);
-    const float yl = __fadd_rn((float)(ty * T), 0.5f), yh = __fadd_rn((float)(ty * T + T), -0.5f);
-    if (hit_q(fminf(fmaxf(u, xl), xh), fminf(fmaxf(v, yl), yh), u, v, ca, cb, cc) <= 9.0f) return true;
-    if (hit_q(xl, fminf(fmaxf(__fadd_rn(v, -__fmul_rn(sy, __fadd_rn(xl, -u))), yl), yh), u, v, ca, cb, cc) <= 9.0f)
-        return true;
-    if (hit_q(xh, fminf(fmaxf(__fadd_rn(v, -__fmul_rn(sy, __fadd_rn(xh, -u))), yl), yh), u, v, ca, cb, cc) <= 9.0f)
-        return true;
-    if (hit_q(fminf(fmaxf(__fadd_rn(u, -__fmul_rn(sx, __fadd_rn(yl, -v))), xl), xh), yl, u, v, ca, cb, cc) <= 9.0f)
-        return true;
-    return hit_q(fminf(fmaxf(__fadd_rn(u, -__fmul_rn(sx, __fadd_rn(yh, -v))), xl), xh), yh, u, v, ca, cb, cc) <= 9.0f;
+                                         int ty, float T) {
+    const float fx = (float)tx, fy = (float)ty, cb2 = __fadd_rn(cb, cb);
+    const float xl = __fmaf_rn(fx, T, 0.5f), xh = __fmaf_rn(fx, T, T - 0.5f);
+    const float yl = __fmaf_rn(fy, T, 0.5f), yh = __fmaf_rn(fy, T, T - 0.5f);
+    const float q0 = hit_q(fminf(fmaxf(u, xl), xh), fminf(fmaxf(v, yl), yh), u, v, ca, cb2, cc);
+    const F2 U = f2(u), V = f2(v), A = f2(ca), B = f2(cb2), D = f2(cc);
+    const F2 ex = sub2(f2(xl, xh), U), ey = sub2(f2(yl, yh), V);
+    const float2 py = un(sub2(V, mul2(f2(sy), ex))), px = un(sub2(U, mul2(f2(sx), ey)));
+    const F2 dy = sub2(f2(fminf(fmaxf(py.x, yl), yh), fminf(fmaxf(py.y, yl), yh)), V);
+    const F2 dx = sub2(f2(fminf(fmaxf(px.x, xl), xh), fminf(fmaxf(px.y, xl), xh)), U);
+    const float2 qx = hit_q2(ex, dy, A, B, D), qy = hit_q2(dx, ey, A, B, D);
+    return q0 <= 9.0f || qx.x <= 9.0f || qx.y <= 9.0f || qy.x <= 9.0f || qy.y <= 9.0f;
+}
+
+// Items of a warp's lanes numbered in lane order, 32 a round: the lanes with items are ranked, the ranks' first
+// numbers are bits of a word per round, and the owner of a lane's item is the rank that the bits up to the
+// lane give.  (A binary search over the lanes' counts by shuffles is five dependent shuffles a round,
+// and another for each value of the owner, which the ranked lanes keep in shared memory instead.)
+struct WarpRuns {
+    uint32_t first;  // number of this lane's first item
+    uint32_t total;  // items of the warp
+    uint32_t rank;   // of this lane among those with items
+    uint32_t before;  // ranks that began in earlier rounds
+    bool any;        // this lane has items
+    __device__ __forceinline__ explicit WarpRuns(uint32_t count) {
+        const uint32_t lane = threadIdx.x & 31;
+        uint32_t incl = count;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (uint32_t)o) incl += t;
+        }
+        total = __shfl_sync(0xffffffffu, incl, 31);
+        first = incl - count;
+        any = count > 0;
+        rank = __popc(__ballot_sync(0xffffffffu, any) & ((1u << lane) - 1u));
+        before = 0;
+    }
+    // rank of the owner of item base + lane (rounds in order, base = 0, 32, ..; the last item's past the end)
+    __device__ __forceinline__ uint32_t owner(uint32_t base) {
+        const uint32_t at = first - base;
+        const uint32_t starts = __reduce_or_sync(0xffffffffu, any && at < 32u ? 1u << at : 0u);
+        const uint32_t o = before + __popc(starts & (0xffffffffu >> (31u - (threadIdx.x & 31)))) - 1u;
+        before += __popc(starts);
+        return o;
+    }
+};
+// local / w for local < 1024, w >= 1 and rw = 1 / w: (local + 1/2) / w is at least 1 / (2 w) from a whole number,
+// its rounding error at most 2^10 / w 2^-22
+__device__ __forceinline__ uint32_t small_quotient(uint32_t local, float rw) {
+    return (uint32_t)__fmul_rn((float)local + 0.5f, rw);
 }
 
 // Reach masks of super-tiles (bit (ty mod kSuperH) kSuperW + tx mod kSuperW = tile (tx, ty)).
