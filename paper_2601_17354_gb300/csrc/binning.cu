@@ -254,79 +254,93 @@ __device__ __forceinline__ uint32_t entry_mask(bool need, uint32_t g, uint2 r, u
 // tiles: read from their reach bits; larger ones whose super-tile rectangle spans at most 2 x 2:
 // the projection's masks; the rest: entry_mask).  Each warp walks
 // the entries of its own 32 Gaussians, 32 per round (entry k by lane k mod 32), whose records it
-// keeps in shared memory by rank.
+// keeps in shared memory by rank.  kEmitWarps warps share the rounds of 32 Gaussians: a round is one
+// chain of dependent steps, and 100k Gaussians are only five warps to each scheduler.  Four where the grid
+// leaves the SMs fewer than four CTAs each, one elsewhere: 100k Gaussians at 1280x720 with 8-pixel tiles (391
+// CTAs) 38 us with one, 26 with two, 22 with four; 200k with 16-pixel tiles (782 CTAs) lose 1 and 10 us
+// a step with two and four, 500k 5 and 25 us (the set-up is most of their work).
 // ---------------------------------------------------------------------------------------------
 struct CoarseRec {
     uint4 a;  // rectangle, hitmask, Gaussian
     uint4 b;  // first entry, super-tiles across | how << 30, super-tiles of a row of the grid, first super-tile
-    uint4 m;  // the projection's masks (how = 0)
+    uint4 m;  // the projection's masks (how = 0), else 1 / super-tiles across (a float)
 };
-__global__ void __launch_bounds__(kProjBlock)
+template <int kEmitWarps>
+__global__ void __launch_bounds__(kProjBlock * kEmitWarps)
 k_coarse_emit(int64_t n, int SX, int T, int64_t capacity, const uint32_t* __restrict__ perm, Scratch sc,
               uint32_t* __restrict__ gidx, uint32_t* __restrict__ gmask, int passes, uint32_t last_mask,
               const RenderDesc* __restrict__ renders, int R) {
     pdl_begin();
     __shared__ CoarseRec s_rec[kProjBlock];
-    __shared__ uint32_t s_warp[kProjBlock / 32];
-    __shared__ BigSmem s_big[kProjBlock / 32];
+    __shared__ uint32_t s_cnt[kProjBlock], s_warp[kProjBlock / 32];
+    __shared__ BigSmem s_big[kProjBlock * kEmitWarps / 32];
     __shared__ uint32_t s_hist[4][kRadix];  // digit counts of the written keys, pass by pass
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, warp = (t & (kProjBlock - 1)) >> 5, part = t / kProjBlock;
     const int64_t i = (int64_t)blockIdx.x * kProjBlock + t;
-    for (int k = t; k < passes * kRadix; k += kProjBlock) (&s_hist[0][0])[k] = 0u;
-    const uint32_t g = i < n ? perm[i] : 0u;
-    const uint32_t reached = i < n ? sc.touched[g] : 0u;
-    uint2 r = make_uint2(0u, 0u);
-    uint32_t cnt = 0, w = 1, how = 0, hm = 0;
-    if (reached) {
-        r = sc.rect[g];
-        uint32_t sx0, sy0, sx1, sy1;
-        super_rect(r, sx0, sy0, sx1, sy1);
-        w = sx1 - sx0;
-        cnt = w * (sy1 - sy0);
-        const uint32_t area = ((r.y & 0xffffu) - (r.x & 0xffffu)) * ((r.y >> 16) - (r.x >> 16));
-        how = area <= 32u ? 1u : w <= 2u && sy1 - sy0 <= 2u ? 0u : 2u;  // hitmask, the projection's masks, entry_mask
-        if (how == 1u) hm = sc.hitmask[g];
-    }
-    WarpRuns runs(cnt);
+    for (int k = t; k < passes * kRadix; k += kProjBlock * kEmitWarps) (&s_hist[0][0])[k] = 0u;
     CoarseRec* const recs = s_rec + 32 * warp;
-    if (reached) {
-        CoarseRec& o = recs[runs.rank];
-        o.a = make_uint4(r.x, r.y, hm, g);
-        uint32_t sx = (uint32_t)SX, first_super = 0;
-        if (renders) {  // batch: item g belongs to the last render whose first item is <= g
-            int lo = 0, hi = R - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (renders[mid].item_base <= (int64_t)g) lo = mid;
-                else hi = mid - 1;
-            }
-            sx = (uint32_t)renders[lo].SX;
-            first_super = (uint32_t)renders[lo].super_base;
+    if (part == 0) {
+        // the Gaussian's record in one memory latency (what a culled one holds there is not used)
+        const uint32_t g = i < n ? perm[i] : 0u;
+        const uint2 r = i < n ? sc.rect[g] : make_uint2(0u, 0u);
+        const uint32_t hm = i < n ? sc.hitmask[g] : 0u;
+        const uint32_t reached = i < n ? sc.touched[g] : 0u;
+        uint32_t cnt = 0, w = 1, how = 0;
+        if (reached) {
+            uint32_t sx0, sy0, sx1, sy1;
+            super_rect(r, sx0, sy0, sx1, sy1);
+            w = sx1 - sx0;
+            cnt = w * (sy1 - sy0);
+            const uint32_t area = ((r.y & 0xffffu) - (r.x & 0xffffu)) * ((r.y >> 16) - (r.x >> 16));
+            how = area <= 32u ? 1u : w <= 2u && sy1 - sy0 <= 2u ? 0u : 2u;  // hitmask, the projection's masks, entry_mask
         }
-        o.b = make_uint4(runs.first, w | (how << 30), sx, first_super);
-        if (how == 0u) o.m = sc.smask[g];
+        s_cnt[t] = cnt;
+        const WarpRuns runs(cnt);
+        if (reached) {
+            CoarseRec& o = recs[runs.rank];
+            o.a = make_uint4(r.x, r.y, hm, g);
+            uint32_t sx = (uint32_t)SX, first_super = 0;
+            if (renders) {  // batch: item g belongs to the last render whose first item is <= g
+                int lo = 0, hi = R - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (renders[mid].item_base <= (int64_t)g) lo = mid;
+                    else hi = mid - 1;
+                }
+                sx = (uint32_t)renders[lo].SX;
+                first_super = (uint32_t)renders[lo].super_base;
+            }
+            o.b = make_uint4(runs.first, w | (how << 30), sx, first_super);
+            if (how == 0u) o.m = sc.smask[g];
+            else o.m.x = __float_as_uint(__frcp_rn((float)w));
+        }
+        if (lane == 0) s_warp[warp] = runs.total;
     }
-    if (lane == 0) s_warp[warp] = runs.total;
-    __syncthreads();  // also publishes the lanes' records in shared memory
+    __syncthreads();
+    const WarpRuns runs(s_cnt[32 * warp + lane]);
     uint32_t before = 0;
 #pragma unroll
     for (int k = 0; k < kProjBlock / 32; ++k) before += k < warp ? s_warp[k] : 0u;
     const unsigned long long out = sc.block_offsets[blockIdx.x] + before;
     uint32_t* ck = reinterpret_cast<uint32_t*>(sc.keys[0]);
-    for (uint32_t b = 0; b < runs.total; b += 32) {  // warp-uniform
+    for (uint32_t b = 32 * part; b < runs.total; b += 32 * kEmitWarps) {  // warp-uniform
         const uint32_t k = b + (uint32_t)lane;
         const CoarseRec& o = recs[runs.owner(b)];
         const bool valid = k < runs.total;
         const uint4 ra = o.a, rb = o.b;
         const uint32_t ow = rb.y & 0x3fffffffu, kind = valid ? rb.y >> 30 : 3u;
-        const uint32_t local = k - rb.x, dy = ow == 1u ? local : local / ow, dx = local - dy * ow;
+        const uint4 rm = o.m;
+        const uint32_t local = k - rb.x;
+        const uint32_t dy = kind == 0u ? local >> (ow - 1u)
+                                       : local < 1024u ? small_quotient(local, __uint_as_float(rm.x)) : local / ow;
+        const uint32_t dx = local - dy * ow;
         const uint32_t sx = (ra.x & 0xffffu) / kSuperW + dx, sy = (ra.x >> 16) / kSuperH + dy;
         const uint2 rect = make_uint2(ra.x, ra.y);
-        uint32_t mask = entry_mask(kind == 2u, ra.w, rect, sx * kSuperW, sy * kSuperH, T, sc, lane, s_big[warp]);
+        uint32_t mask = entry_mask(kind == 2u, ra.w, rect, sx * kSuperW, sy * kSuperH, T, sc, lane, s_big[t >> 5]);
         if (kind == 1u)
             mask = super_mask_from_hits(ra.z, rect.x & 0xffffu, rect.x >> 16, rect.y & 0xffffu, rect.y >> 16, sx, sy);
         else if (kind == 0u)
-            mask = smask_slot(o.m, 2u * dy + dx);
+            mask = smask_slot(rm, 2u * dy + dx);
         const unsigned long long pos = out + k;
         if (valid && pos < (unsigned long long)capacity) {
             const uint32_t key = rb.w + sy * rb.z + sx;
@@ -341,7 +355,7 @@ k_coarse_emit(int64_t n, int SX, int T, int64_t capacity, const uint32_t* __rest
     // the sort's digit totals: this CTA's counts added into its partial copy (zeroed before)
     __syncthreads();
     uint32_t* copy = sc.digit_totals + (blockIdx.x % kTotalCopies) * (kMaxPasses * kRadix);
-    for (int k = t; k < passes * kRadix; k += kProjBlock) {
+    for (int k = t; k < passes * kRadix; k += kProjBlock * kEmitWarps) {
         const uint32_t v = (&s_hist[0][0])[k];
         if (v) atomicAdd(&copy[k], v);
     }
@@ -841,24 +855,26 @@ k_seg_scan(int64_t capacity, uint32_t* __restrict__ wc, Scratch sc) {
 }
 
 // The pairs of every block (values = canonical indices into out), and the ranges of a super-tile's
-// tiles from its first block.  Per warp and round the 32 masks are transposed, so lane x holds the
-// set of lanes reaching tile x: its count is one popcount and an entry's rank among them another.
+// tiles from its first block.  Tile by tile, the warp's lanes whose entries reach it write side by side: an
+// entry's pairs written by its own lane go to a line each, 32 different ones an instruction, and
+// the lane with the most tiles holds its warp (39 us for the 6.5 M pairs of 500k Gaussians at
+// 1920x1080, 27 us now; put together in shared memory first and written in runs of a block, 50 us).
 __global__ void __launch_bounds__(kFineThreads)
 k_fine_emit(int64_t capacity, int TX, int TY, const uint32_t* __restrict__ cv, const uint32_t* __restrict__ gidx,
             const uint32_t* __restrict__ gmask, const uint32_t* __restrict__ wc, int S, uint32_t* __restrict__ out,
             Scratch sc, const RenderDesc* __restrict__ renders, int R) {
     pdl_begin();
-    __shared__ uint32_t s_cw[kFineWarps][32];
-    __shared__ uint32_t s_off[kFineWarps][32];
+    __shared__ uint32_t s_cw[kFineWarps * kFineRounds][32];
+    __shared__ __align__(16) uint32_t s_off[kFineWarps * kFineRounds][32];  // of a warp's round, tile by tile
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
+    const uint32_t cap = capacity < 0xffffffffll ? (uint32_t)capacity : 0xffffffffu;
     const uint32_t VB = sc.vbase[S];
     for (uint32_t v = blockIdx.x; v < VB; v += gridDim.x) {
         if ((uint64_t)v >= (uint64_t)capacity / 32) break;
         const uint4 bi = sc.binfo[v];
         const uint32_t s = bi.x;
-        uint32_t g[kFineRounds], m[kFineRounds], col[kFineRounds];
-        uint32_t cnt = 0;
+        uint32_t g[kFineRounds], m[kFineRounds];
 #pragma unroll
         for (int r = 0; r < kFineRounds; ++r) {
             const uint64_t e = (uint64_t)bi.y + warp * (32 * kFineRounds) + r * 32 + lane;
@@ -868,11 +884,8 @@ k_fine_emit(int64_t capacity, int TX, int TY, const uint32_t* __restrict__ cv, c
             m[r] = valid ? gmask[e0] : 0u;
         }
 #pragma unroll
-        for (int r = 0; r < kFineRounds; ++r) {
-            col[r] = warp_transpose(m[r], lane);  // lanes whose entry of round r reaches tile `lane`
-            cnt += __popc(col[r]);
-        }
-        s_cw[warp][lane] = cnt;
+        for (int r = 0; r < kFineRounds; ++r)  // lanes whose entry of round r reaches tile `lane`
+            s_cw[warp * kFineRounds + r][lane] = __popc(warp_transpose(m[r], lane));
         __syncthreads();
         if (warp == 0) {
             const uint32_t tt = sc.stt[32 * s + lane];
@@ -885,7 +898,7 @@ k_fine_emit(int64_t capacity, int TX, int TY, const uint32_t* __restrict__ cv, c
             const uint32_t ts = sc.sbase[s] + incl - tt;  // the tile's first pair
             uint32_t base = ts + wc[32ull * v + lane];
 #pragma unroll
-            for (int w = 0; w < kFineWarps; ++w) {
+            for (int w = 0; w < kFineWarps * kFineRounds; ++w) {
                 s_off[w][lane] = base;
                 base += s_cw[w][lane];
             }
@@ -893,30 +906,24 @@ k_fine_emit(int64_t capacity, int TX, int TY, const uint32_t* __restrict__ cv, c
                 const SuperCell c = super_cell(s, TX, TY, renders, R);
                 const uint32_t tx = c.sx * kSuperW + (lane % kSuperW), ty = c.sy * kSuperH + (lane / kSuperW);
                 if ((int)tx < c.TX && (int)ty < c.TY) {
-                    const uint32_t cap = capacity < 0xffffffffll ? (uint32_t)capacity : 0xffffffffu;
                     sc.ranges[c.tile_base + ty * (uint32_t)c.TX + tx] = make_uint2(min(ts, cap), min(ts + tt, cap));
                 }
             }
         }
         __syncthreads();
-        // each lane writes its entries' pairs: tile x after the warp's earlier entries that reach x
+#pragma unroll 2
+        for (int x0 = 0; x0 < 32; x0 += 4)
 #pragma unroll
-        for (int r = 0; r < kFineRounds; ++r) {
-            uint32_t mm = m[r];
-            const int rounds = __reduce_max_sync(kFull, (uint32_t)__popc(mm));
-            for (int it = 0; it < rounds; ++it) {  // warp-uniform
-                const int x = mm ? __ffs(mm) - 1 : 0;
-                uint32_t earlier = 0;
+            for (int r = 0; r < kFineRounds; ++r) {
+                const uint4 off = *reinterpret_cast<const uint4*>(&s_off[warp * kFineRounds + r][x0]);
+                const uint32_t at[4] = {off.x, off.y, off.z, off.w};
 #pragma unroll
-                for (int q = 0; q < r; ++q) earlier += __popc(__shfl_sync(kFull, col[q], x));
-                const uint32_t cx = __shfl_sync(kFull, col[r], x);
-                if (mm) {
-                    const uint64_t pos = (uint64_t)s_off[warp][x] + earlier + __popc(cx & lt);
-                    if (pos < (uint64_t)capacity) out[pos] = g[r];
-                    mm &= mm - 1u;
+                for (int k = 0; k < 4; ++k) {
+                    const bool in = (m[r] >> (x0 + k)) & 1u;
+                    const uint32_t pos = at[k] + __popc(__ballot_sync(kFull, in) & lt);
+                    if (in && pos < cap) out[pos] = g[r];
                 }
             }
-        }
         __syncthreads();
     }
 }
@@ -1164,8 +1171,9 @@ int launch_bin_lists(int64_t n, int TX, int TY, int T, int64_t tiles, int64_t su
     const uint32_t last_mask = passes > 0 ? (uint32_t)((1u << (bits - kRadixBits * (passes - 1))) - 1u) : 0u;
     if (!cleared) cudaMemsetAsync(sc.digit_totals, 0, sizeof(uint32_t) * kTotalWords, s);
     if (nb > 0) {
-        launch_pdl(k_coarse_emit, dim3(nb), dim3(kProjBlock), 0, s, n, (TX + kSuperW - 1) / kSuperW, T, capacity, perm,
-                   sc, gidx, gmask, passes, last_mask, renders, R);
+        const bool few = nb < 4 * 152;
+        launch_pdl(few ? k_coarse_emit<4> : k_coarse_emit<1>, dim3(nb), dim3(kProjBlock * (few ? 4 : 1)), 0, s, n,
+                   (TX + kSuperW - 1) / kSuperW, T, capacity, perm, sc, gidx, gmask, passes, last_mask, renders, R);
         ++launched;
     }
     // the coarse entries arrive in depth order: a stable sort by super-tile keeps it in each

@@ -379,7 +379,6 @@ struct WarpRuns {
     uint32_t first;  // number of this lane's first item
     uint32_t total;  // items of the warp
     uint32_t rank;   // of this lane among those with items
-    uint32_t before;  // ranks that began in earlier rounds
     bool any;        // this lane has items
     __device__ __forceinline__ explicit WarpRuns(uint32_t count) {
         const uint32_t lane = threadIdx.x & 31;
@@ -393,15 +392,13 @@ struct WarpRuns {
         first = incl - count;
         any = count > 0;
         rank = __popc(__ballot_sync(0xffffffffu, any) & ((1u << lane) - 1u));
-        before = 0;
     }
-    // rank of the owner of item base + lane (rounds in order, base = 0, 32, ..; the last item's past the end)
-    __device__ __forceinline__ uint32_t owner(uint32_t base) {
+    // rank of the owner of item base + lane (the last item's past the end)
+    __device__ __forceinline__ uint32_t owner(uint32_t base) const {
         const uint32_t at = first - base;
         const uint32_t starts = __reduce_or_sync(0xffffffffu, any && at < 32u ? 1u << at : 0u);
-        const uint32_t o = before + __popc(starts & (0xffffffffu >> (31u - (threadIdx.x & 31)))) - 1u;
-        before += __popc(starts);
-        return o;
+        const uint32_t before = __popc(__ballot_sync(0xffffffffu, any && first < base));
+        return before + __popc(starts & (0xffffffffu >> (31u - (threadIdx.x & 31)))) - 1u;
     }
 };
 // local / w for local < 1024, w >= 1 and rw = 1 / w: (local + 1/2) / w is at least 1 / (2 w) from a whole number,
