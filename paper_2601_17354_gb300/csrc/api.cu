@@ -102,7 +102,7 @@ size_t carve_g(Scratch& sc, char* base, int64_t n, int64_t pixels, int64_t tiles
     sc.pair_count = c.take<unsigned long long>(1);
     sc.pair_need = c.take<unsigned long long>(1);
     sc.coarse_count = c.take<unsigned long long>(1);
-    sc.bin_ticket = c.take<uint32_t>(3);
+    sc.bin_ticket = c.take<uint32_t>(2);
     sc.tile_buckets = c.take<uint32_t>(256);
     sc.sort_blocks = c.take<uint32_t>(1);
     sc.digit_totals = c.take<uint32_t>(kTotalWords);
@@ -343,7 +343,6 @@ static int render_impl(pgs_ctx* ctx, const pgs_gaussians* params, const pgs_came
     const size_t e2 = mark(ctx);
     ctx->launches += launch_bin_lists(params->n, TX, TY, T, tiles, supers, ctx->cap_pairs, perm, ctx->sc, s, &ctx->buf,
                                       nullptr, 0, cleared);
-    ctx->launches += launch_tile_order((int)tiles, ctx->sc, s);
     const size_t e3 = mark(ctx);
     ctx->recorded = false;
     if (ctx->replay_k > 0) {
@@ -812,7 +811,6 @@ int64_t enqueue_render(pgs_batch* b) {
     k += launch_bin_count(b->items, b->supers, b->cap_pairs, perm, b->sc, s);
     k += launch_bin_lists(b->items, 0, 0, b->cfg.tile, b->tiles, b->supers, b->cap_pairs, perm, b->sc, s, &b->buf,
                           b->d_renders, b->R);
-    k += launch_tile_order((int)b->tiles, b->sc, s);
     return k;
 }
 

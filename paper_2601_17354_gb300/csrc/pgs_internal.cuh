@@ -122,7 +122,7 @@ struct Scratch {
     unsigned long long* pair_count = nullptr;
     unsigned long long* pair_need = nullptr;  // pair capacity the render needs (>= pair_count)
     unsigned long long* coarse_count = nullptr;
-    uint32_t* bin_ticket = nullptr;  // [3] arrival counters of the binning's last-CTA steps (reset by it)
+    uint32_t* bin_ticket = nullptr;  // [2] arrival counters of the binning's last-CTA steps (reset by it)
     uint32_t* tile_buckets = nullptr;  // [256] tile-order bucket counts (kept zero between renders), cursors
     uint32_t* sort_blocks = nullptr;  // sort CTAs with work in the current render
     uint32_t* digit_totals = nullptr; // [kTotalCopies][kMaxPasses][kRadix]
@@ -292,10 +292,6 @@ int launch_radix_sort_only(int64_t capacity, int key_bits, const Scratch& sc, cu
 // Failure-detection self-test: one sort pass whose first tile is never published (the next tile's
 // bounded wait runs out and records kStatusTimeout); needs a pair capacity of three sort tiles.
 int launch_timeout_selftest(int64_t capacity, const Scratch& sc, cudaStream_t s);
-
-// Order the tiles by decreasing list length (quarter-octave buckets), so the compositing grids
-// start the heaviest tiles first.
-int launch_tile_order(int tiles, const Scratch& sc, cudaStream_t s);
 
 // K6/K8: compositing forward and backward (sorted values in buffer `buf`).
 // The L1 loss fused into the compositing forward (target == nullptr: off): with n = 3 H W values,
