@@ -434,7 +434,7 @@ constexpr size_t scatter_smem() { return (sizeof(KeyT) + sizeof(uint32_t)) * kTh
 // and only the first kRadix threads take the per-digit steps (their own named barrier)
 template <typename KeyT, int kItems, int kThreads = kSortThreads>
 __global__ void __launch_bounds__(kThreads)
-k_onesweep(int64_t capacity, int pass, int shift, uint32_t dmask, int sb_max, const KeyT* __restrict__ kin,
+k_onesweep(int64_t capacity, int pass, int shift, uint32_t dmask, int sb_max, bool spare, const KeyT* __restrict__ kin,
            const uint32_t* __restrict__ vin, KeyT* __restrict__ kout, uint32_t* __restrict__ vout, Scratch sc) {
     pdl_begin();
     static_assert(kThreads % kRadix == 0, "whole digit warps");
@@ -451,30 +451,48 @@ k_onesweep(int64_t capacity, int pass, int shift, uint32_t dmask, int sb_max, co
     __shared__ uint32_t s_part[kDigitWarps];
     __shared__ uint32_t s_hist[kRadix];            // the tile's count of digit d
     __shared__ uint32_t s_tile;
+    __shared__ int s_gone;  // a wait ran out
     uint32_t* head = sc.sort_hist;  // [0] abort word, [1 + pass] ticket of the pass, then the look-back
     uint32_t* lb = sc.sort_hist + kLookbackHead + (size_t)pass * kRadix * sb_max;
+    // A pass over few tiles is a chain of memory latencies, so everything it reads is asked for at once: the
+    // digit totals (needed last), and the keys of the tile that the ticket most likely names (CTAs are started in
+    // order).  2,000 keys took 9.6 us a pass with each waiting for the one before, 7.4 us now; 500k
+    // keys 13.5 us, 12.6 us.  A grid sized for the capacity has CTAs to spare (eight in nine of the 2,395 for the
+    // super-tile sort of 500k Gaussians): those leave first, the tiles are for the others.
     const uint32_t nblk = *sc.sort_blocks;
+    if (spare && blockIdx.x >= nblk) return;
     if (threadIdx.x == 0) s_tile = atomicAdd(&head[1 + pass], 1u);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = threadIdx.x; k < kWarps * kRadix; k += kThreads) (&s_wh[0][0])[k] = 0;
-    if (threadIdx.x < kRadix) s_hist[threadIdx.x] = 0;
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    if (tile >= nblk) return;
     const uint64_t P = kept_pairs(sc, capacity);
-    const uint64_t cbase = (uint64_t)tile * kTile;
-    const uint64_t wbase = cbase + (uint64_t)warp * kWarpItems;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     KeyT key[kRounds];
     uint32_t val[kRounds];
     uint32_t dr[kRounds];  // digit | warp-local rank << 8
+    auto load_tile = [&](uint32_t t) {
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-        const uint64_t idx = wbase + (uint64_t)r * 32 + lane;
-        const bool valid = idx < P;
-        key[r] = valid ? kin[idx] : (KeyT)0;
-        val[r] = valid ? vin[idx] : 0u;
+        for (int r = 0; r < kRounds; ++r) {
+            const uint64_t idx = (uint64_t)t * kTile + (uint64_t)warp * kWarpItems + (uint64_t)r * 32 + lane;
+            const bool valid = idx < P;
+            key[r] = valid ? kin[idx] : (KeyT)0;
+            val[r] = valid ? vin[idx] : 0u;
+        }
+    };
+    load_tile(blockIdx.x);
+    uint32_t total[kTotalCopies];
+    if (threadIdx.x < kRadix) {
+#pragma unroll
+        for (int cpy = 0; cpy < kTotalCopies; ++cpy)
+            total[cpy] = sc.digit_totals[pass * kRadix + (size_t)cpy * kMaxPasses * kRadix + threadIdx.x];
     }
+    for (int k = threadIdx.x; k < kWarps * kRadix; k += kThreads) (&s_wh[0][0])[k] = 0;
+    if (threadIdx.x < kRadix) s_hist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_gone = 0;
+    __syncthreads();
+    const uint32_t tile = s_tile;
+    if (tile >= nblk) return;
+    if (tile != blockIdx.x) load_tile(tile);
+    const uint64_t cbase = (uint64_t)tile * kTile;
+    const uint64_t wbase = cbase + (uint64_t)warp * kWarpItems;
     // the tile's digit counts, published before the ranking
 #pragma unroll
     for (int r = 0; r < kRounds; ++r)
@@ -520,6 +538,7 @@ k_onesweep(int64_t capacity, int pass, int shift, uint32_t dmask, int sb_max, co
             // kLbWindow predecessors per round, loaded together: the walk over tiles that have
             // published only their count costs one memory latency per window, not per tile
             int spins = 0;
+            bool gone = false;
             int64_t t = (int64_t)tile - 1;
             while (t >= 0) {
                 uint32_t w[kLbWindow];
@@ -550,15 +569,18 @@ k_onesweep(int64_t capacity, int pass, int shift, uint32_t dmask, int sb_max, co
                     if ((spins & 63) == 0 && ld_relaxed(head) != 0u) break;  // another wait ran out
                     __nanosleep(64);
                 }
-                if (ld_relaxed(head) != 0u) break;
+                if (ld_relaxed(head) != 0u) {
+                    gone = true;
+                    break;
+                }
             }
-            st_relaxed(mine, kLbPrefix | (before + acc));
+            if (gone) s_gone = 1;  // and no prefix: the tiles after this one end at the same wait
+            else st_relaxed(mine, kLbPrefix | (before + acc));
         }
         // offset of digit d in the pass's output: all keys of smaller digits + the tiles before
-        const uint32_t* tot = sc.digit_totals + pass * kRadix;
         uint32_t all = 0;
 #pragma unroll
-        for (int cpy = 0; cpy < kTotalCopies; ++cpy) all += tot[(size_t)cpy * kMaxPasses * kRadix + d];
+        for (int cpy = 0; cpy < kTotalCopies; ++cpy) all += total[cpy];
         uint32_t incl_all = all, incl = acc;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -583,7 +605,7 @@ k_onesweep(int64_t capacity, int pass, int shift, uint32_t dmask, int sb_max, co
         s_bstart[d] = wpre + incl - acc;
     }
     __syncthreads();
-    if (ld_relaxed(head) != 0u) return;  // a wait ran out: the pass is abandoned (status recorded)
+    if (s_gone) return;  // a wait of this tile ran out: its keys stay where they were (status recorded)
 #pragma unroll
     for (int r = 0; r < kRounds; ++r) {
         if (dr[r] != 0xffffffffu) {
@@ -1015,10 +1037,11 @@ static int super_bits(int64_t supers) {
     return bits;
 }
 
-// cleared: the look-back words (and, unless totals_ready, the digit totals) are already zero.
+// cleared: the look-back words (and, unless totals_ready, the digit totals) are already zero.  spare: there may be
+// fewer keys than the capacity.
 template <typename KeyT, int kItems, int kThreads = kSortThreads>
 int sort_passes(int64_t capacity, int first_shift, int bits, const Scratch& sc, cudaStream_t s, int* out_buf,
-                bool totals_ready = false, bool cleared = false) {
+                bool totals_ready = false, bool cleared = false, bool spare = true) {
     constexpr int kTile = kThreads * kItems;
     const int passes = (bits + kRadixBits - 1) / kRadixBits;
     const uint32_t last_mask = passes > 0 ? (uint32_t)((1u << (bits - kRadixBits * (passes - 1))) - 1u) : 0u;
@@ -1042,7 +1065,7 @@ int sort_passes(int64_t capacity, int first_shift, int bits, const Scratch& sc, 
         const int shift = first_shift + p * kRadixBits;
         const uint32_t dmask = p == passes - 1 ? last_mask : (uint32_t)(kRadix - 1);
         launch_pdl(k_onesweep<KeyT, kItems, kThreads>, dim3(sb_max), dim3(kThreads), scatter_smem<KeyT, kItems, kThreads>(),
-                   s, capacity, p, shift, dmask, sb_max, (const KeyT*)k[buf], (const uint32_t*)sc.vals[buf], k[buf ^ 1],
+                   s, capacity, p, shift, dmask, sb_max, spare, (const KeyT*)k[buf], (const uint32_t*)sc.vals[buf], k[buf ^ 1],
                    sc.vals[buf ^ 1], sc);
         buf ^= 1;
     }
@@ -1068,7 +1091,7 @@ int launch_timeout_selftest(int64_t capacity, const Scratch& sc, cudaStream_t s)
     uint32_t* k0 = reinterpret_cast<uint32_t*>(sc.keys[0]);
     uint32_t* k1 = reinterpret_cast<uint32_t*>(sc.keys[1]);
     k_onesweep<uint32_t, kSortItems><<<2, kSortThreads, scatter_smem<uint32_t, kSortItems>(), s>>>(
-        capacity, 0, 0, kRadix - 1, sb_max, k0, sc.vals[0], k1, sc.vals[1], sc);
+        capacity, 0, 0, kRadix - 1, sb_max, false, k0, sc.vals[0], k1, sc.vals[1], sc);
     return 2;
 }
 
@@ -1083,7 +1106,7 @@ int launch_depth_sort(int64_t n, const Scratch& sc, cudaStream_t s, const uint32
     d.pair_count = sc.dcount;
     d.sort_blocks = sc.dblocks;
     int buf = 0;
-    const int launched = sort_passes<uint32_t, kDepthItems, kDepthThreads>(n, 0, 32, d, s, &buf, false, cleared);
+    const int launched = sort_passes<uint32_t, kDepthItems, kDepthThreads>(n, 0, 32, d, s, &buf, false, cleared, false);
     *perm = sc.dvals[buf];
     return launched;
 }
