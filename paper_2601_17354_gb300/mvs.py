@@ -13,7 +13,7 @@ import numpy as np
 import torch
 
 from . import _lib as L
-from .rasterizer import camera_struct
+from .rasterizer import camera_array, camera_struct
 
 
 def _p(t: torch.Tensor) -> C.c_void_p:
@@ -62,7 +62,7 @@ class MultiViewStereo:
 
     def select_reference(self, cams, target: int, median_depth: float):
         """(reference index, scores [len(cams)]) by Eq. 4."""
-        arr = (L.PgsCamera * len(cams))(*[camera_struct(c) for c in cams])
+        arr = camera_array(cams)
         scores = np.zeros(len(cams), np.float64)
         ref = C.c_int32()
         L.check(self._lib.pgs_mvs_select_reference(self._m, arr, len(cams), int(target), float(median_depth),
