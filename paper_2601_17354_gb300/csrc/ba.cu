@@ -370,8 +370,7 @@ k_ba_linearize(int64_t n, int C, const float* __restrict__ R, const float* __res
             float r[2], iz, w;
             cam_point_df(R, t, i, px, py, pz, X);
             float4* __restrict__ H = Htp + 5 * o;
-            const float2 q = reinterpret_cast<const float2*>(uv)[o];
-            if (!residual(X, K, q.x, q.y, rb, r, iz, w, rho)) {
+            if (!residual(X, K, uv[2 * o], uv[2 * o + 1], rb, r, iz, w, rho)) {
                 for (int k = 0; k < 5; ++k) H[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                 continue;
             }
@@ -1055,9 +1054,8 @@ k_ba_backsub(int64_t n, const int64_t* __restrict__ start, const int32_t* __rest
         for (int64_t o = o0 + l; o < o1; o += kGroup) {
             Df X[3], rho;
             float r[2], iz, w;
-            const float2 q = reinterpret_cast<const float2*>(uv)[o];
             cam_point_df(Rn, tn, cam[o], pn[0], pn[1], pn[2], X);
-            if (residual(X, K, q.x, q.y, rb, r, iz, w, rho)) df_acc(rho_sum, rho);
+            if (residual(X, K, uv[2 * o], uv[2 * o + 1], rb, r, iz, w, rho)) df_acc(rho_sum, rho);
             else df_acc(rho_sum, 1e30f);
         }
     }
