@@ -9,10 +9,10 @@
 // d2 = fma(dx, dx, fma(dy, dy, dz * dz)) with dx = p_j - p_i, ties broken by index, so the neighbour
 // lists are reproducible bit for bit.  The bounding box and the grid stay on the device.
 //
-// Features and the paper's initializer are computed per point at about twice FP32's precision: Eq. 5
-// covariance of the K_n = 16 nearest neighbours about their centroid, its smallest-eigenvalue
-// eigenvector as the normal (cyclic Jacobi, eigenvectors canonicalised so the largest-magnitude
-// component is positive), Eq. 6 tangential scale from the K_s = 3 nearest neighbours, normal scale
+// Features and the paper's initializer are computed per point at about twice FP32's precision, in FP64 where that
+// does not decide (k_features_init): Eq. 5 covariance of the K_n = 16 nearest neighbours about their centroid, its
+// smallest-eigenvalue eigenvector as the normal (cyclic Jacobi, eigenvectors canonicalised so the
+// largest-magnitude component is positive), Eq. 6 tangential scale from the K_s = 3 nearest neighbours, normal scale
 // r_normal s_t, z axis rotated onto the normal, opacity logit(0.1); and the 16 features of the
 // learned initializer from the 32 nearest neighbours.
 #include <cuda_bf16.h>
@@ -26,10 +26,6 @@ namespace pgs {
 namespace {
 
 constexpr int kThreads = 256;
-
-// Order-preserving integer image of a float (and its own inverse): non-negative floats keep their
-// bits, negative ones flip all but the sign bit, so signed integer order = float order.
-__device__ __host__ __forceinline__ int ordered(int bits) { return bits >= 0 ? bits : bits ^ 0x7fffffff; }
 
 struct Grid {
     float lo[3];
@@ -423,6 +419,63 @@ __device__ void jacobi3(const Df a[6], Df w[3], Df V[3][3]) {
     }
 }
 
+// w (times scale^2) and V of the covariance of the first k neighbours [neighbour][axis][point] in FP64, for a
+// point whose eigenvalues lie too close for two floats (see k_features_init).
+struct Frame {
+    Df w[3], V[3][3];
+};
+__device__ __noinline__ Frame frame64(const float (*nb)[3][33], int point, int k, double scale) {
+    double c[3] = {0, 0, 0}, A[3][3] = {}, U[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
+    for (int a = 0; a < k; ++a)
+        for (int d = 0; d < 3; ++d) c[d] += (double)nb[a][d][point];
+    for (int d = 0; d < 3; ++d) c[d] /= k;
+    for (int a = 0; a < k; ++a) {
+        double v[3];
+        for (int d = 0; d < 3; ++d) v[d] = (double)nb[a][d][point] - c[d];
+        for (int x = 0; x < 3; ++x)
+            for (int y = 0; y < 3; ++y) A[x][y] += v[x] * v[y];
+    }
+    for (int x = 0; x < 3; ++x)
+        for (int y = 0; y < 3; ++y) A[x][y] /= k;
+    for (int sweep = 0; sweep < 64; ++sweep) {
+        if (A[0][1] * A[0][1] + A[0][2] * A[0][2] + A[1][2] * A[1][2] < 1e-300) break;
+        for (int p = 0; p < 2; ++p)
+            for (int q = p + 1; q < 3; ++q) {
+                if (A[p][q] == 0.0) continue;
+                const double theta = (A[q][q] - A[p][p]) / (2.0 * A[p][q]);
+                const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+                const double co = 1.0 / sqrt(t * t + 1.0), si = t * co;
+                auto turn = [&](double& f, double& g) {
+                    const double h = co * f - si * g;
+                    g = si * f + co * g;
+                    f = h;
+                };
+                for (int r = 0; r < 3; ++r) turn(A[r][p], A[r][q]);
+                for (int r = 0; r < 3; ++r) turn(A[p][r], A[q][r]);
+                for (int r = 0; r < 3; ++r) turn(U[r][p], U[r][q]);
+            }
+    }
+    int at[3] = {0, 1, 2};  // columns by ascending eigenvalue
+    for (int e = 0; e < 3; ++e) {
+        const int i = e == 1 ? 1 : 0;
+        if (A[at[i + 1]][at[i + 1]] < A[at[i]][at[i]]) {
+            const int t = at[i];
+            at[i] = at[i + 1];
+            at[i + 1] = t;
+        }
+    }
+    Frame f;
+    for (int j = 0; j < 3; ++j) {
+        const int from = at[j];
+        int big = 0;
+        for (int r = 1; r < 3; ++r)
+            if (fabs(U[r][from]) > fabs(U[big][from])) big = r;
+        f.w[j] = df_from(A[from][from] * scale * scale);
+        for (int r = 0; r < 3; ++r) f.V[r][j] = df_from(U[big][from] < 0 ? -U[r][from] : U[r][from]);
+    }
+    return f;
+}
+
 __device__ void mat_to_quat(const double R[3][3], double q[4]) {
     const double tr = R[0][0] + R[1][1] + R[2][2];
     if (tr > 0) {
@@ -458,9 +511,11 @@ __device__ void mat_to_quat(const double R[3][3], double q[4]) {
 // neighbours into shared memory, a point's 32 at a time (one coalesced read of its list), for the two
 // passes over them.  Offsets from the point are exact in two floats and are scaled by a power of two to
 // about 1.  In FP64 throughout, 200k points took 3.33 ms, all of it in the FP64 pipe; FP64 is left
-// where a handful of values a point leave the kernel through a logarithm or a quaternion.  0.39 ms now, with
-// one copy of the eigenvalue code for both neighbourhoods (expanded twice, the code outgrew the
-// instruction cache: 0.46 ms) and one pass over the neighbours for both covariances.
+// where a handful of values a point leave the kernel through a logarithm or a quaternion, and for neighbourhoods
+// that two floats do not decide (of 200k points on a sphere or a plane none, on one line all: 568 us for 2,000
+// points in FP64 throughout, 552 here).  0.36 to 0.38 ms now (on a plane the extra pass for the smallest eigenvalue
+// is 0.01 of it), with one copy of the eigenvalue code for both neighbourhoods (expanded twice, the code
+// outgrew the instruction cache: 0.46 ms) and one pass over the neighbours for both covariances.
 constexpr int kFeatWarps = 2;
 __global__ void __launch_bounds__(32 * kFeatWarps)
 k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restrict__ nb, float r_normal,
@@ -477,14 +532,16 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
     __syncwarp();
     if (i >= n) return;
     const float p0[3] = {P[i], P[n + i], P[2 * n + i]};
-    // scale: the farthest neighbour's offset has its largest component in [1, 2)
+    // scale: the farthest neighbour's offset has its largest component in [1, 2); the coordinates are scaled
+    // before the difference, which then neither overflows nor rounds
     float far = 0.f;
-    for (int d = 0; d < 3; ++d) far = fmaxf(far, fabsf(s_nb[warp][31][d][lane] - p0[d]));
-    const int ex = far > 0.f && far < 1e30f ? max(ilogbf(far), -100) : 0;
+    for (int d = 0; d < 3; ++d) far = fmaxf(far, fabsf(0.5f * s_nb[warp][31][d][lane] - 0.5f * p0[d]));
+    const int ex = far > 0.f && isfinite(far) ? min(max(ilogbf(far) + 1, -100), 127) : 0;
     const float scale = ldexpf(1.0f, -ex);
+    const float q0[3] = {p0[0] * scale, p0[1] * scale, p0[2] * scale};
     auto offset = [&](int a, Df u[3]) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) u[d] = df_scale(df_two(s_nb[warp][a][d][lane], -p0[d]), scale);
+        for (int d = 0; d < 3; ++d) u[d] = df_two(s_nb[warp][a][d][lane] * scale, -q0[d]);
     };
     // sums of the offsets (the first 16, all 32) and of the distances (the first 3, all 32)
     const Df zero = {0.f, 0.f};
@@ -508,44 +565,46 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
     }
     settle(d3);
     settle(d32);
-    // covariances (times 16 and 32) about the 32 neighbours' mean rounded to FP32 in one pass; what the
-    // true means differ by is taken out after
-    float c32[3];
+    // covariances (times 16 and 32), each about its own mean: the 16 nearest about theirs, moved to the mean of
+    // all 32 by adding 16 e e^T, then the rest about that.  (Taken about one centre and corrected by a
+    // subtraction, the covariance of 16 neighbours that lie close together drowns in the rounding of the other's.)
+    Df c[3], e[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) c32[d] = m32[d].h * 0.03125f;
-    Df C16[6] = {zero, zero, zero, zero, zero, zero}, C32[6] = {zero, zero, zero, zero, zero, zero};
+    for (int d = 0; d < 3; ++d) {
+        c[d] = df_scale(m16[d], 0.0625f);
+        m32[d] = df_scale(m32[d], 0.03125f);  // the means from here on
+        e[d] = df_sub(c[d], m32[d]);
+    }
+    Df C16[6], C32[6] = {zero, zero, zero, zero, zero, zero};
 #pragma unroll 1
     for (int a = 0; a < 32; ++a) {
-        Df u[3], v[3];
-        offset(a, u);
-        if (a == 16)
+        Df v[3];
+        offset(a, v);
+        if (a == 16) {
+            int k = 0;
 #pragma unroll
-            for (int e = 0; e < 6; ++e) C16[e] = C32[e];
+            for (int x = 0; x < 3; ++x) {
+                c[x] = m32[x];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const Df t = df_two(u[d].h, -c32[d]);
-            v[d] = df_fast(t.h, __fadd_rn(t.l, u[d].l));
+                for (int y = x; y < 3; ++y, ++k) {
+                    C16[k] = df_two(C32[k].h, C32[k].l);
+                    C32[k] = df_add(C16[k], df_scale(df_mul(e[x], e[y]), 16.0f));
+                }
+            }
         }
-        int e = 0;
 #pragma unroll
-        for (int x = 0; x < 3; ++x)
-#pragma unroll
-            for (int y = x; y < 3; ++y) df_dot(C32[e++], v[x], v[y]);
-    }
-    // C - k e e^T, e = mean - centre; the division by k scales exactly
-    auto finish = [&](Df C[6], const Df m[3], float inv) {
-        Df e[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) e[d] = df_add(df_scale(m[d], inv), {-c32[d], 0.f});
+        for (int d = 0; d < 3; ++d) v[d] = df_sub(v[d], c[d]);
         int k = 0;
 #pragma unroll
         for (int x = 0; x < 3; ++x)
 #pragma unroll
-            for (int y = x; y < 3; ++y, ++k)
-                C[k] = df_sub(df_scale(df_two(C[k].h, C[k].l), inv), df_mul(e[x], e[y]));
-    };
-    finish(C32, m32, 0.03125f);
-    finish(C16, m16, 0.0625f);
+            for (int y = x; y < 3; ++y) df_dot(C32[k++], v[x], v[y]);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        C16[k] = df_scale(C16[k], 0.0625f);
+        C32[k] = df_scale(df_two(C32[k].h, C32[k].l), 0.03125f);
+    }
     // both decompositions through one copy of the code: it and the loops above are several times the
     // instruction cache when expanded
     Df w[3], V[3][3], nrm[3];
@@ -553,11 +612,50 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
     for (int pass = 0; pass < 2; ++pass) {
         Df C[6];
 #pragma unroll
-        for (int e = 0; e < 6; ++e) C[e] = pass ? C32[e] : C16[e];
+        for (int k = 0; k < 6; ++k) C[k] = pass ? C32[k] : C16[k];
         jacobi3(C, w, V);
+        // An eigenvector is known to 3e-14 of the trace over its distance from the next eigenvalue.  Below 4e-6 of
+        // the trace that is no longer far under FP32's rounding; nor does it settle an eigenvector's sign when its
+        // two largest components are that close, and nothing is known of points closer together than 1e-10 of
+        // the farthest offset.  Such neighbourhoods (lines, lattices, coincident points) take FP64.
+        const float trace = w[0].h + w[1].h + w[2].h, close = 4e-6f * trace;
+        bool open = !(w[1].h - w[0].h > close) || (pass && !(w[2].h - w[1].h > close)) || !(trace > 1e-20f);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float x = fabsf(V[0][k].h), y = fabsf(V[1][k].h), z = fabsf(V[2][k].h), xy = fmaxf(x, y);
+            const float second = fmaxf(fminf(x, y), fminf(xy, z));
+            open = open || ((k == 0 || pass) && !(fmaxf(xy, z) - second > 1e-7f));
+        }
+        if (open) {
+            const Frame fr = frame64(s_nb[warp], lane, pass ? 32 : 16, scale);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                w[a] = fr.w[a];
+#pragma unroll
+                for (int b = 0; b < 3; ++b) V[a][b] = fr.V[a][b];
+            }
+        }
         if (pass == 0)  // the smallest eigenvector of the 16 neighbours: the normal
 #pragma unroll
             for (int d = 0; d < 3; ++d) nrm[d] = V[d][0];
+    }
+    if (w[0].h < 4e-6f * w[2].h) {
+        // A flat neighbourhood: the covariance knows its smallest eigenvalue to 1e-14 of the trace only.  The mean
+        // square of the offsets along the normal, which cancels nothing, has it to FP32 however small.
+        Df at = zero, sq = zero;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) df_dot(at, V[d][0], m32[d]);
+        at = df_two(at.h, at.l);
+#pragma unroll 1
+        for (int a = 0; a < 32; ++a) {
+            Df u[3], t = zero;
+            offset(a, u);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) df_dot(t, V[d][0], u[d]);
+            t = df_sub(df_two(t.h, t.l), at);
+            df_dot(sq, t, t);
+        }
+        w[0] = df_scale(df_two(sq.h, sq.l), 0.03125f);
     }
     float f[16];
     const Df sum = df_add(df_add(w[0], w[1]), w[2]);
@@ -568,7 +666,7 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
 #pragma unroll
         for (int d = 0; d < 3; ++d) f[3 + 3 * k + d] = V[d][k].h;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) f[12 + d] = df_ratio(m32[d], d32);
+    for (int d = 0; d < 3; ++d) f[12 + d] = df_ratio(m32[d], df_scale(d32, 0.03125f));
     const double unit = ldexp(1.0, ex);
     f[15] = (float)(-3.0 * log(df_double(d32) * (0.03125 * unit)));
 #pragma unroll
