@@ -1,5 +1,7 @@
 // C ABI of the bundle adjustment (kernels in ba.cu, contract in include/pocketgs.h).
+#include <algorithm>
 #include <cmath>
+#include <memory>
 #include <new>
 
 #include "pgs_internal.cuh"
@@ -209,15 +211,18 @@ int pgs_ba_solve(pgs_ba* b, float* R, float* t, float* P, const int32_t* cam, co
     int axis = 0;
     int rc = begin(b, R, t, cam, pt, &axis);
     if (rc != PGS_OK) return rc;
-    if (iters + 1 > b->costs_cap) {
+    const int64_t rows = (int64_t)iters + 1;
+    std::unique_ptr<double[]> got(new (std::nothrow) double[(size_t)rows]);
+    if (!got) return PGS_ERR_OOM;
+    if (rows > b->costs_cap) {
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return err(e);
         if (b->costs) cudaFree(b->costs);
         b->costs = nullptr;
         b->costs_cap = 0;
-        e = cudaMalloc(&b->costs, sizeof(double) * ((size_t)iters + 1));
+        e = cudaMalloc(&b->costs, sizeof(double) * (size_t)rows);
         if (e != cudaSuccess) return err(e);
-        b->costs_cap = (int64_t)iters + 1;
+        b->costs_cap = rows;
     }
     // the whole solve is enqueued; the device accepts or rejects each candidate
     const Problem q{cam, pt, uv, K, sigma, huber_delta};
@@ -233,9 +238,11 @@ int pgs_ba_solve(pgs_ba* b, float* R, float* t, float* P, const int32_t* cam, co
     if (rc != PGS_OK) return rc;
     BaCtl ctl{};
     cudaError_t e = cudaMemcpyAsync(&ctl, b->ctl, sizeof(ctl), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(costs, b->costs, sizeof(double) * ((size_t)iters + 1), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(got.get(), b->costs, sizeof(double) * (size_t)rows, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return err(e);
+    // a solve that stopped has costs up to its last decision only; the caller's others stay as they are
+    std::copy(got.get(), got.get() + (ctl.stop ? ctl.it + 1 : rows), costs);
     if (ctl.stop) return PGS_ERR_NOT_PD;
     *accepted = ctl.accepted;
     return PGS_OK;
