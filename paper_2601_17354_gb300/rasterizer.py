@@ -83,13 +83,16 @@ def tensors_struct(n, sh_degree, means, log_scales, quats, opacity_logits, sh) -
 
 
 def camera_struct(cam) -> L.PgsCamera:
+    return _camera_struct(cam, [float(b) for b in getattr(cam, "bg", (0.0, 0.0, 0.0))])
+
+
+def _camera_struct(cam, bg) -> L.PgsCamera:
     vm = np.ascontiguousarray(cam.viewmat, np.float32).reshape(-1)
     # one copy of the twelve values where there are twelve (8 us a camera value by value, 3 us so)
     view = (C.c_float * 12).from_buffer_copy(vm) if vm.size == 12 else (C.c_float * 12)(*vm.tolist())
-    bg = getattr(cam, "bg", (0.0, 0.0, 0.0))
     return L.PgsCamera(int(cam.width), int(cam.height), float(cam.fx), float(cam.fy),
                        float(cam.cx), float(cam.cy), view,
-                       float(getattr(cam, "near", 0.2)), (C.c_float * 3)(*[float(b) for b in bg]))
+                       float(getattr(cam, "near", 0.2)), (C.c_float * 3)(*bg))
 
 
 _CAMERA = np.dtype([("size", "<u4", 2), ("k", "<f4", 4), ("view", "<f4", 12), ("near", "<f4"), ("bg", "<f4", 3)])
@@ -97,11 +100,13 @@ _CAMERA = np.dtype([("size", "<u4", 2), ("k", "<f4", 4), ("view", "<f4", 12), ("
 
 def camera_array(cams):
     """camera_struct of every camera, as one C array: column by column (64 cameras one by one took
-    0.56 ms, more than a keyframe's depth map on the GPU; 0.12 ms so)."""
+    0.56 ms, more than a keyframe's depth map on the GPU; 0.12 ms so).  The cameras and their backgrounds may be
+    anything that can be gone through once."""
+    cams = list(cams)
     views = [np.asarray(c.viewmat, np.float32).reshape(-1) for c in cams]
-    bgs = [getattr(c, "bg", (0.0, 0.0, 0.0)) for c in cams]
+    bgs = [[float(b) for b in getattr(c, "bg", (0.0, 0.0, 0.0))] for c in cams]
     if not views or any(v.size != 12 for v in views) or any(len(b) != 3 for b in bgs):
-        return (L.PgsCamera * len(cams))(*[camera_struct(c) for c in cams])
+        return (L.PgsCamera * len(cams))(*[_camera_struct(c, b) for c, b in zip(cams, bgs)])
     arr = (L.PgsCamera * len(cams))()
     out = np.frombuffer(arr, _CAMERA)
     with np.errstate(over="ignore"):  # a value beyond FP32 becomes infinite, as in a C float
@@ -109,7 +114,7 @@ def camera_array(cams):
         out["k"] = [(float(c.fx), float(c.fy), float(c.cx), float(c.cy)) for c in cams]
         out["view"] = views
         out["near"] = [float(getattr(c, "near", 0.2)) for c in cams]
-        out["bg"] = [[float(v) for v in b] for b in bgs]
+        out["bg"] = bgs
     return arr
 
 
