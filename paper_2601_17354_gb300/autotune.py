@@ -1,13 +1,15 @@
 """Autotuner of the rasterizer: picks the screen tile edge (8, 16, 32 pixels), the pixels-per-thread
 strip (1, 2, 4) and the number of list entries staged in shared memory per batch (64, 128, 256) by
 timing them on the caller's own workload (every variant's forward + backward compositing, and per
-tile edge the render part of the step), and caches the choices in a JSON file keyed by GPU and
+tile edge the render part of the step), and caches the choices in a JSON file keyed by GPU, kernels and
 workload class (batch shape, resolution class, Gaussian count), so later runs skip the timing."""
 from __future__ import annotations
 
+import functools
 import json
 import math
 import os
+import zlib
 from dataclasses import dataclass
 
 import torch
@@ -41,8 +43,19 @@ def resolution_class(width: int, height: int) -> str:
     return f"{width}x{height}"
 
 
+@functools.lru_cache(maxsize=None)
+def _kernels() -> str:
+    """Which kernels a stored choice was timed on: a checksum of the sources of what is timed (compositing, and for
+    the tile edge the projection and binning)."""
+    crc = 0
+    for name in ("composite.cu", "project.cu", "binning.cu"):
+        with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc", name), "rb") as f:
+            crc = zlib.crc32(f.read(), crc)
+    return f"{crc:08x}"
+
+
 def workload_key(kind: str, resolutions, n_gaussians: int, sh_degree: int) -> str:
-    gpu = torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu"
+    gpu = (torch.cuda.get_device_name() if torch.cuda.is_available() else "cpu") + " " + _kernels()
     res = "+".join(sorted(set(resolutions)))
     return f"{gpu}|{kind}|{res}|N~2^{round(math.log2(max(n_gaussians, 1)))}|sh{sh_degree}"
 
