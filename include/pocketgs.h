@@ -370,7 +370,7 @@ void pgs_init_destroy(pgs_init* ctx);
 /* The k (3, 16 or 32) nearest other points of each of n points [3][n] (device fp32): nb [n][k]
    (device int32), ascending by squared distance d2 = fma(dx,dx, fma(dy,dy, dz*dz)) in fp32 with
    ties by index; exact (uniform grid, search widened until provably complete).  -1 pads when
-   n - 1 < k.  Synchronises once (bounding box). */
+   n - 1 < k.  Synchronises only when its scratch grows. */
 int pgs_knn(pgs_init* ctx, const float* points, int64_t n, int32_t k, int32_t* nb);
 
 /* From 32-neighbour lists nb [n][32]: the paper's initializer (Eq. 5 normal from 16 neighbours,
@@ -422,8 +422,9 @@ int pgs_make_targets(pgs_init* ctx, const pgs_gaussians* pca, const pgs_gaussian
    Bundle adjustment of the geometry prior (Sec. III-A): Levenberg-Marquardt on the robust
    reprojection objective (Eq. 2), each step solved through the reduced camera system (Eq. 3):
    the point blocks are inverted independently (3 x 3 each), folded into a dense 6C x 6C camera
-   system (Schur complement), which is solved by Cholesky (FP64), and the point steps follow by
-   back-substitution.
+   system (Schur complement), which is scaled to a unit diagonal and solved by Cholesky in FP32,
+   and the point steps follow by back-substitution.  Residuals, costs, the point blocks and their
+   inverses carry 46 bits or more; the arrays need the alignment of their elements only.
      camera i: world-to-camera rotation R_i (row-major 3 x 3) and translation t_i, x = R_i P + t_i;
      observation o of point pt[o] in camera cam[o] at pixel uv[o]; intrinsics K = (fx, fy, cx, cy);
      residual r = pi(x) - uv, whitened norm e = |r| / sigma; Huber: rho = e^2 (e <= delta) or
@@ -455,15 +456,18 @@ int pgs_ba_step(pgs_ba* ba, const float* R, const float* t, const float* P, cons
 /* `iters` Levenberg-Marquardt trials from lambda0, R, t, P updated in place: a trial whose
    robust cost is lower is taken and lambda divided by 10, else lambda multiplied by 10 and the
    linearization reused.  costs [iters + 1] (host) receives the cost after each trial (costs[0]
-   initial), *accepted (host) the number taken.  Synchronises once per trial. */
+   initial), *accepted (host) the number taken.  The trials are enqueued together and synchronise
+   once at their end.  On PGS_ERR_NOT_PD the state is that of the last trial taken, costs holds the
+   costs up to the last decision and *accepted is not written. */
 int pgs_ba_solve(pgs_ba* ba, float* R, float* t, float* P, const int32_t* cam, const int32_t* pt,
                  const float* uv, const float* K, float sigma, float huber_delta, int32_t iters,
                  float lambda0, double* costs, int32_t* accepted);
 
 /* Device times (ms) of the stages of one iteration from the given state (nothing applied):
    ms[0] point linearization (H_pp, b_p, H_tp), ms[1] camera blocks (H_tt, b_t), ms[2] point
-   inverses and E, ms[3] reduced-system blocks, ms[4] reduced-system solve, ms[5]
-   back-substitution and candidate poses, ms[6] candidate cost.  Synchronises. */
+   inverses, ms[3] reduced-system blocks, ms[4] assembly and solve of the reduced system and
+   candidate poses, ms[5] back-substitution and the candidate's cost, ms[6] the decision on that
+   cost.  Synchronises. */
 int pgs_ba_stage_times(pgs_ba* ba, const float* R, const float* t, const float* P, const int32_t* cam,
                        const int32_t* pt, const float* uv, const float* K, float sigma, float huber_delta,
                        float lambda, float* ms);

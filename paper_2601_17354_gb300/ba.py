@@ -1,7 +1,7 @@
 """Bundle adjustment of the geometry prior (Sec. III-A) on the GPU: Levenberg-Marquardt on the
 robust reprojection objective of Eq. 2, each step solved through the reduced camera system of
-Eq. 3 (independent 3 x 3 point inverses, dense FP64 Cholesky of the 6C x 6C camera system,
-back-substitution of the points).
+Eq. 3 (independent 3 x 3 point inverses, FP32 Cholesky of the 6C x 6C camera system scaled to a unit
+diagonal, back-substitution of the points).
 
 Cameras are world-to-camera (R [C][3][3], t [C][3]); points P [n][3]; observations (cam, pt, uv)
 grouped by point (pt non-decreasing); intrinsics (fx, fy, cx, cy).  All arithmetic runs in
@@ -100,6 +100,7 @@ class BundleAdjuster:
                                        C.byref(acc)), "pgs_ba_solve")
         return costs, int(acc.value)
 
+    # "solve" includes the candidate poses, "backsub" the candidate's cost; "cost" is the decision on it
     STAGES = ["linearize", "camblocks", "points", "schur", "solve", "backsub", "cost"]
 
     def stage_times(self, R, t, P, cam, pt, uv, K, sigma: float, delta: float, lam: float):

@@ -527,8 +527,9 @@ __device__ __forceinline__ void pair_alpha(F2 dy, F2 DX, F2 ADX2, F2 S2Y, F2 S2Z
 // are evaluated together: only the transmittance chains them, and a tile with few warps beside it
 // waits on latency.  The composited count of two pixels shares one word: an entry takes at
 // least 1/255 of T and T stays over 1e-4, so no pixel composites more than 2,346 entries.
-// Measured (256 staged): 500k Gaussians at 1920x1080 0.241 -> 0.220 ms, 61k at 1237x693 0.070 -> 0.062,
-// 2k at 128x128 27 -> 24 us; one or two entries at a time take 0.258-0.266 ms at 1920x1080.  The wider
+// Measured (256 staged, the launch alone and repeated): 500k Gaussians at 1920x1080 0.241 -> 0.222 ms, 61k at
+// 1237x693 0.070 -> 0.062, 2k at 128x128 27 -> 24 us; in a training step, with the fused loss and cold caches, 0.251 ->
+// 0.236 ms at 1920x1080.  One or two entries at a time take 0.258-0.266 ms there.  The wider
 // staging costs 8-pixel tiles their occupancy at 256 staged entries (0.080 -> 0.092 ms at 100k and
 // 1280x720), which is why theirs is 64 (0.061).
 template <int kT, int kPix, int kDepth>
@@ -1608,8 +1609,10 @@ __global__ void k_trace_pixels(int W, int H, int TX, int T, int64_t n, const uin
 //            64 / 128 / 256, backward 0.131 / 0.153 / 0.227)
 //   edge 16  forward 256 (500k, 1920x1080: 0.226 / 0.220 / 0.220), backward 128 (0.451 / 0.447 / 0.499;
 //            61k, 1237x693: 0.125 / 0.125 / 0.145)
-//   edge 32  256 (not measured apart)
-// A batch has one depth for both directions: the backward's, the longer one.
+//   edge 32  256 both ways (500k, 1920x1080: forward 0.445 / 0.419 / 0.405, backward 0.909 / 0.903 / 0.850; 200k,
+//            1280x720: 0.321 / 0.308 / 0.295, 0.534 / 0.521 / 0.505)
+// A batch has one depth for both directions: the backward's, the longer one (with 16-pixel tiles its forward loses
+// nothing by 128: 0.222 / 0.222 at 500k, 0.061 / 0.062 at 61k).
 // PGS_COMPOSITE_PIXELS / PGS_COMPOSITE_DEPTH override all of them (read once per process).
 CompositeVariant default_variant(int T, bool backward) {
     static const CompositeVariant env = [] {

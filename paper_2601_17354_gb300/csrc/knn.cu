@@ -231,7 +231,8 @@ __device__ __forceinline__ unsigned long long exchange(unsigned long long k, int
 
 // The K nearest other points of each point, a warp per point.  Instruction-bound: 32 candidates cost
 // about 40 instructions to fetch and rate, a batch with more than kFew candidates among the best so far
-// one bitonic sort and merge (21 exchanges), fewer of them an insertion each.  A thread per point
+// one bitonic sort and merge (21 exchanges), fewer of them an insertion each (200k points on a plane: 408 us for
+// the whole search at kFew = 4, 402 at 10, 436 at 20; on a sphere 324, 322, 333).  A thread per point
 // with its list in registers paid a pass of 32 compare-and-swaps whenever any lane of its warp had
 // a candidate and walked cells one by one: 200k surface points, K = 32, 2.35 ms.
 constexpr int kQueryWarps = 4;

@@ -75,8 +75,8 @@ __device__ __forceinline__ void frag_a_t(uint32_t a[4], const __nv_bfloat16* S, 
 __device__ __forceinline__ F2 phi2(F2 z, F2& e) {
     const F2 x = mul2(z, f2(0.70710678118654752f));
     const float2 xv = un(x);
-    // ex2 and rcp with flushed subnormals: the arguments of rcp are at least 1, and e^{-x^2} below 2^-126
-    // changes no activation's sum
+    // ex2 and rcp with flushed subnormals: the arguments of rcp are at least 1, and where e^{-x^2} is below 2^-126
+    // (z < -13.2) the activation, itself below 2e-37, becomes zero.  Keeping those costs 471 -> 539 us at 6.4 M points.
     const float2 w = un(mul2(mul2(x, x), f2(-1.4426950408889634f)));
     F2 s;
     {

@@ -139,7 +139,8 @@ k_census(const float* __restrict__ rgb_t, const float* __restrict__ rgb_r, int W
 __device__ __forceinline__ int floor_fast(float q, bool& sure) {
     const float m = __fadd_rn(q, -0.5f), t = __fadd_rn(m, 12582912.0f);
     const float d = __fadd_rn(m, -__fadd_rn(t, -12582912.0f));
-    // (also false for |q| over 2^18 and for NaN)
+    // (the margin is used up from |q| = 499,998 on, and by NaN; below that the sums are exact to the rounding the
+    // margin allows for, 1.5 2^23 holding integers to 2^22)
     sure = sure && fabsf(d) < __fmaf_rn(fabsf(q), -1e-6f, 0.499998f);
     return __float_as_int(t) - 0x4b400000;
 }

@@ -134,9 +134,11 @@ k_ssim_fwd(const float* __restrict__ img, const float* __restrict__ tgt, int W, 
             const float2 mu = un(m1[j]), sq = un(m2[j]);
             const float mx = mu.x, my = mu.y;
             const float sxx = sq.x - mx * mx, syy = sq.y - my * my, sxyc = m12[j] - mx * my;
+            // sxx + syy is a difference of filtered moments and may come out below zero on flat patches, by about 1e-7 of the
+            // squared values: B2 stays positive, C2 = 9e-4, for images of values of order one
             const float A1 = 2.f * mx * my + kC1, A2 = 2.f * sxyc + kC2;
             const float B1 = mx * mx + my * my + kC1, B2 = sxx + syy + kC2;
-            const float rb1 = __fdividef(1.0f, B1), rb2 = __fdividef(1.0f, B2);  // B1, B2 >= C1, C2 > 0
+            const float rb1 = __fdividef(1.0f, B1), rb2 = __fdividef(1.0f, B2);  // B1 >= C1; B2: see above
             const float inv = rb1 * rb2;
             const float s = A1 * A2 * inv;
             const float ds_dmu = 2.f * my * A2 * inv - s * 2.f * mx * rb1;  // sigmas held fixed
