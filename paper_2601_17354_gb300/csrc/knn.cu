@@ -619,16 +619,16 @@ k_features_init(int64_t n, const float* __restrict__ P, const int32_t* __restric
         for (int k = 0; k < 6; ++k) C[k] = pass ? C32[k] : C16[k];
         jacobi3(C, w, V);
         // An eigenvector is known to 3e-14 of the trace over its distance from the next eigenvalue.  Below 4e-6 of
-        // the trace that is no longer far under FP32's rounding; nor does it settle an eigenvector's sign when its
-        // two largest components are that close, and nothing is known of points closer together than 1e-10 of
-        // the farthest offset.  Such neighbourhoods (lines, lattices, coincident points) take FP64.
+        // the trace that is no longer far under FP32's rounding; nor does it settle an eigenvector's sign when two
+        // components of opposite sign are its largest to 3e-8, and nothing is known of points closer together than
+        // 1e-10 of the farthest offset.  Such neighbourhoods (lines, lattices, coincident points) take FP64: about
+        // 12 us to the launch where one warp in 200k points has one.
         const float trace = w[0].h + w[1].h + w[2].h, close = 4e-6f * trace;
         bool open = !(w[1].h - w[0].h > close) || (pass && !(w[2].h - w[1].h > close)) || !(trace > 1e-20f);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float x = fabsf(V[0][k].h), y = fabsf(V[1][k].h), z = fabsf(V[2][k].h), xy = fmaxf(x, y);
-            const float second = fmaxf(fminf(x, y), fminf(xy, z));
-            open = open || ((k == 0 || pass) && !(fmaxf(xy, z) - second > 1e-7f));
+        for (int k = 0; k < 3; ++k) {  // (the largest component is positive: the sign hangs on a negative one near it)
+            const float big = fmaxf(V[0][k].h, fmaxf(V[1][k].h, V[2][k].h));
+            open = open || ((k == 0 || pass) && !(big + fminf(V[0][k].h, fminf(V[1][k].h, V[2][k].h)) > 3e-8f));
         }
         if (open) {
             const Frame fr = frame64(s_nb[warp], lane, pass ? 32 : 16, scale);
